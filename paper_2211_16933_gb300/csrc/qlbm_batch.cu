@@ -173,50 +173,88 @@ static cudaError_t launch_stage(ql_batch *b, int stage, int warps, int grid, boo
     return fm ? launch_fm_all(b) : cudaSuccess;
 }
 
-// Fields of every instance averaged over blocks of nx/ncoarse cells:
-// out[(i * 5 + f) * ncoarse + c] for f = rho, u, T, q, Pxx.  One thread per
-// (instance, coarse cell); moments per fine cell in FP64 (Sec. II.D).
+// double(x) by integer arithmetic, exact (also for denormal x): the conversion
+// instruction occupies the FP64 pipe, which bounds the kernel below.
+__device__ __forceinline__ double to_double_(float x)
+{
+    const bool sub = (__float_as_uint(x) & 0x7F800000u) == 0;
+    const uint32_t v = __float_as_uint(sub ? x * 4294967296.0f : x), e = (v >> 23) & 0xFFu;
+    const uint32_t hi = (v & 0x80000000u) | ((e == 255u ? 2047u : e + (sub ? 864u : 896u)) << 20) | ((v >> 3) & 0xFFFFFu);
+    return (v << 1) == 0 ? 0.0 : __hiloint2double(int(hi), int(v << 29));
+}
+__device__ __forceinline__ double to_double_(double x) { return x; }
+
+// Fields of every instance averaged over blocks of f = nx/ncoarse cells:
+// out[(i * 5 + f) * ncoarse + c] for f = rho, u, T, q, Pxx; moments per fine
+// cell in FP64 (Sec. II.D), from the sums and differences of the mirrored
+// velocities.  FP64 arithmetic bounds it (about 5 instructions per velocity; one
+// pass over the state would take a tenth of that).  One thread per fine cell, so
+// that a warp reads consecutive cells of a row (one thread per coarse cell, the
+// form before, walked f cells each with strides of f between the lanes: 2687 us
+// for 256 instances of 256 - 8192 cells and 64 coarse cells): a block takes
+// 256 / f whole coarse cells of blockIdx.y's instance, or one coarse cell of more
+// than 256 in several turns, and sums each in a fixed order: kFieldParts strided
+// partial sums, then those in turn.
+constexpr int kFieldThreads = 256, kFieldParts = 8;
 template <typename Real>
-__global__ void batch_fields_kernel(const BatchInstance *__restrict__ inst, const void *__restrict__ arena,
-                                    const double *__restrict__ tab, int ncoarse, double *__restrict__ out)
+__global__ void __launch_bounds__(kFieldThreads)
+    batch_fields_kernel(const BatchInstance *__restrict__ inst, const void *__restrict__ arena,
+                        const double *__restrict__ tab, int ncoarse, double *__restrict__ out)
 {
     using V = typename std::conditional<sizeof(Real) == 4, float2, double2>::type;
-    const int i = blockIdx.y;
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= ncoarse) return;
-    const BatchInstance I = inst[i];
-    const int Q = I.Q;
-    int p_off = 0;
-    switch (Q) {
-    case 8: p_off = tab_view(8).p; break;
-    case 16: p_off = tab_view(16).p; break;
-    case 24: p_off = tab_view(24).p; break;
-    default: p_off = tab_view(32).p; break;
-    }
-    const V *psi = static_cast<const V *>(arena) + I.off;
+    __shared__ double s_v[5][kFieldThreads];
+    __shared__ double s_p[5][kFieldThreads];  // partial sums [5][coarse cell][part] (at most 32 coarse cells), then running sums
+    const BatchInstance &I = inst[blockIdx.y];
     const int64_t f = I.nx / ncoarse;
-    double acc[5] = {0, 0, 0, 0, 0};
-    for (int64_t j = 0; j < f; ++j) {
-        const int64_t cell = int64_t(c) * f + j;
-        double S0 = 0, S1 = 0, S2 = 0, S3 = 0, R0 = 0, R1 = 0;
-        for (int k = 0; k < Q; ++k) {
-            const V v = psi[int64_t(k) * I.stride + kHalo + cell];
-            const double ph = double(v.x), th = double(v.y), p = tab[p_off + k];
-            S0 += ph;
-            S1 += p * ph;
-            S2 += p * p * ph;
-            S3 += p * p * p * ph;
-            R0 += th;
-            R1 += p * th;
+    // whole coarse cells per block: the partial sums of one field fit kFieldThreads
+    const int per = int(f > kFieldThreads ? 1 : (kFieldThreads / f < kFieldThreads / kFieldParts ? kFieldThreads / f : kFieldThreads / kFieldParts));
+    const int64_t c0 = int64_t(blockIdx.x) * per;
+    if (c0 >= ncoarse) return;  // the whole block
+    const int nc = int(ncoarse - c0 < per ? ncoarse - c0 : per);
+    const int Q = I.Q, H = Q / 2, t = threadIdx.x;
+    const double *p = tab + (Q == 8 ? tab_view(8).p : Q == 16 ? tab_view(16).p : Q == 24 ? tab_view(24).p : tab_view(32).p) + H;
+    const V *psi = static_cast<const V *>(arena) + I.off + kHalo + c0 * f;
+    const int64_t stride = I.stride, cells = nc * f;
+    for (int64_t b0 = 0; b0 < cells; b0 += kFieldThreads) {
+        const int n = int(cells - b0 < kFieldThreads ? cells - b0 : kFieldThreads);
+        if (t < n) {
+            double S0 = 0, S1 = 0, S2 = 0, S3 = 0, R0 = 0, R1 = 0;
+#pragma unroll 4
+            for (int j = 0; j < H; ++j) {
+                const V va = psi[int64_t(H + j) * stride + b0 + t], vb = psi[int64_t(H - 1 - j) * stride + b0 + t];
+                const double fa = to_double_(va.x), fb = to_double_(vb.x), ta = to_double_(va.y), tb = to_double_(vb.y);
+                const double pj = p[j], sm = fa + fb, d1 = pj * (fa - fb), p2 = pj * pj;
+                S0 += sm;
+                S1 += d1;
+                S2 = fma(p2, sm, S2);
+                S3 = fma(p2, d1, S3);
+                R0 += ta + tb;
+                R1 = fma(pj, ta - tb, R1);
+            }
+            const double u = S1 / S0, c2 = fma(-u, S1, S2);
+            s_v[0][t] = S0;
+            s_v[1][t] = u;
+            s_v[2][t] = (c2 + R0) / (3.0 * S0);
+            s_v[3][t] = 0.5 * (S3 - 3.0 * u * S2 + 2.0 * u * u * S1 + R1 - u * R0);
+            s_v[4][t] = c2;
         }
-        const double n = S0, u = S1 / n, c2 = S2 - u * S1;
-        acc[0] += n;
-        acc[1] += u;
-        acc[2] += (c2 + R0) / (3.0 * n);
-        acc[3] += 0.5 * (S3 - 3.0 * u * S2 + 2.0 * u * u * S1 + R1 - u * R0);
-        acc[4] += c2;
+        __syncthreads();
+        // partial sum `part` of coarse cell c (of this turn's cells when f > kFieldThreads)
+        const int len = f > kFieldThreads ? n : int(f), work = nc * kFieldParts;
+        for (int e = t; e < 5 * work; e += kFieldThreads) {
+            const int q = e / work, r = e - q * work, c = r / kFieldParts, part = r - c * kFieldParts;
+            double acc = b0 > 0 ? s_p[q][r] : 0.0;
+            for (int j = part; j < len; j += kFieldParts) acc += s_v[q][c * len + j];
+            s_p[q][r] = acc;
+        }
+        __syncthreads();
     }
-    for (int q = 0; q < 5; ++q) out[(int64_t(i) * 5 + q) * ncoarse + c] = acc[q] / double(f);
+    for (int e = t; e < 5 * nc; e += kFieldThreads) {
+        const int q = e / nc, c = e - q * nc;
+        double acc = 0.0;
+        for (int k = 0; k < kFieldParts; ++k) acc += s_p[q][c * kFieldParts + k];
+        out[(int64_t(blockIdx.y) * 5 + q) * ncoarse + c0 + c] = acc / double(f);
+    }
 }
 
 // Sec. IV.A: amplitude of density mode m of every instance,
@@ -624,11 +662,14 @@ ql_status ql_batch_fields(ql_batch *b, int32_t ncoarse, double *out)
     for (int64_t i = 0; i < b->n; ++i)
         if (b->inst[i].nx % ncoarse != 0)
             return bfail(b, QL_EINVAL, "ncoarse must divide nx of every instance (instance " + std::to_string(i) + ")");
-    const dim3 grid(unsigned((ncoarse + 127) / 128), unsigned(b->n));
+    // blocks of the instance with the most cells per coarse cell (the others' surplus blocks return at once)
+    const int64_t f = b->max_nx / ncoarse;
+    const int64_t per = std::max<int64_t>(1, std::min<int64_t>(kFieldThreads / kFieldParts, kFieldThreads / f));
+    const dim3 grid(unsigned((ncoarse + per - 1) / per), unsigned(b->n));
     if (b->precision == QL_FP32)
-        batch_fields_kernel<float><<<grid, 128, 0, b->stream>>>(b->d_inst, b->arena[0], b->d_tab64, ncoarse, out);
+        batch_fields_kernel<float><<<grid, kFieldThreads, 0, b->stream>>>(b->d_inst, b->arena[0], b->d_tab64, ncoarse, out);
     else
-        batch_fields_kernel<double><<<grid, 128, 0, b->stream>>>(b->d_inst, b->arena[0], b->d_tab64, ncoarse, out);
+        batch_fields_kernel<double><<<grid, kFieldThreads, 0, b->stream>>>(b->d_inst, b->arena[0], b->d_tab64, ncoarse, out);
     QB_CUDA(b, cudaGetLastError());
     return QL_OK;
 }
