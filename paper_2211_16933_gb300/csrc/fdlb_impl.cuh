@@ -2,6 +2,9 @@
 // this file a unit defines QL_REAL (float or double), QL_SUFFIX (f32 or f64)
 // and declares `static __constant__ QL_REAL QL_TAB[kTabTotal]`.
 #pragma once
+#include <math.h>
+#include <string.h>
+
 #include "fdlb_kernels.cuh"
 #include "fdlb_aux.cuh"
 
@@ -30,6 +33,27 @@ cudaError_t QL_FN(upload_tables_)(const double *all)
             host[tv.cb + l] = QL_REAL(l >= 2 ? l - 1 : 0);
         }
     }
+#ifdef QL_LOGTAB
+    // interval j of log_<double>: high words 0x3FE6A000 + j 2^13 up, c_j its middle (1 for the two next
+    // to 1); leading parts are multiples of 2^-42
+    static double2 lt[258];
+    auto split = [](long double v, double *h, double *l) {
+        *h = rint(double(v) * 4398046511104.0) / 4398046511104.0;
+        *l = double(v - (long double)*h);
+    };
+    for (int j = 0; j < 128; ++j) {
+        const uint64_t lo = uint64_t(0x3FE6A000u + (unsigned(j) << 13)) << 32, hi = lo + (uint64_t(1) << 45);
+        double a, b;
+        memcpy(&a, &lo, 8);
+        memcpy(&b, &hi, 8);
+        const bool one = a == 1.0 || b == 1.0;
+        lt[2 * j].x = one ? 1.0 : 2.0 / (a + b);
+        split(one ? 0.0L : -logl((long double)lt[2 * j].x), &lt[2 * j].y, &lt[2 * j + 1].x);
+    }
+    split(0.693147180559945309417232121458176568L, &lt[257].x, &lt[257].y);
+    const cudaError_t e = cudaMemcpyToSymbol(QL_LOGTAB, lt, sizeof(lt));
+    if (e != cudaSuccess) return e;
+#endif
     return cudaMemcpyToSymbol(QL_TAB, host, sizeof(host));
 }
 

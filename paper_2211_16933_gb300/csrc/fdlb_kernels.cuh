@@ -21,6 +21,7 @@
 #include <stdint.h>
 
 #include "qlbm_internal.h"
+#include "weno_i64.cuh"
 
 namespace qlbm {
 
@@ -70,22 +71,65 @@ __device__ __forceinline__ double2 sub2(double2 a, double2 b) { return make_doub
 // small fraction of the FP32 rate on this GPU).
 __device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
-__device__ __forceinline__ float max_(float a, float b) { return fmaxf(a, b); }
-__device__ __forceinline__ double max_(double a, double b) { return fmax(a, b); }
 
-template <typename Real>
-__device__ __forceinline__ Real rsqrt_(Real x);
-template <>
-__device__ __forceinline__ float rsqrt_<float>(float x) { return rsqrtf(x); }
-template <>
-__device__ __forceinline__ double rsqrt_<double>(double x) { return rsqrt(x); }
+// sqrt(x) for normal x > 0.  FP64: from the hardware's reciprocal square root r0
+// (PTX rsqrt.approx.ftz.f64), x r0 (1 + e/2 + 3 e^2/8) with e = 1 - x r0^2.
+__device__ __forceinline__ float sqrt_(float x) { return x * rsqrtf(x); }
+__device__ __forceinline__ double sqrt_(double x)
+{
+    double r;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double t = x * r, e = fma(-t, r, 1.0);
+    return fma(t * e, fma(0.375, e, 0.5), t);
+}
+// x > 0, and x finite, without FP64 comparisons (each holds the FP64 pipe as long as a multiplication).
+__device__ __forceinline__ bool positive_(float x) { return x > 0.f; }
+__device__ __forceinline__ bool positive_(double x)
+{
+    const int hi = __double2hiint(x);
+    return (hi > 0 || (hi == 0 && __double2loint(x) != 0)) && hi <= 0x7FF00000 &&
+           !(hi == 0x7FF00000 && __double2loint(x) != 0);
+}
+__device__ __forceinline__ bool finite_(float x) { return isfinite(x); }
+__device__ __forceinline__ bool finite_(double x) { return (__double2hiint(x) & 0x7FF00000) != 0x7FF00000; }
 
 template <typename Real>
 __device__ __forceinline__ Real log_(Real x);
 template <>
 __device__ __forceinline__ float log_<float>(float x) { return logf(x); }
+// FP64: the library's log takes 32 FP64 instructions (2083 cycles per warp
+// measured), this 15: table-driven reduction (P. T. P. Tang, ACM TOMS 16, 1990)
+// x = 2^e m with m in [0.707, 1.414), m = c (1 + r) with c at the middle of one of
+// 128 intervals (c = 1 on the two next to 1), |r| < 2^-7, and the Taylor series of
+// log(1 + r) to r^8.  e log 2 + log c is held in two parts, the leading one exact
+// (multiples of 2^-42), so the result is within 0.6 units in the last place.  For
+// finite normal x > 0; others give NaN.
+#ifdef QL_LOGTAB
+template <>
+__device__ __forceinline__ double log_<double>(double x)
+{
+    const int hi = __double2hiint(x);
+    if (unsigned(hi - 0x00100000) >= 0x7FE00000u) return __hiloint2double(0x7FF80000, 0);
+    const int d = hi - 0x3FE6A000;
+    const int e = d >> 20, j = (d >> 13) & 127;
+    const double m = __hiloint2double(hi - (e << 20), __double2loint(x));
+    const double2 t = QL_LOGTAB[2 * j];  // 1 / c, leading part of log c
+    const double r = fma(m, t.x, -1.0), r2 = r * r;
+    double p = fma(r, -1.0 / 8.0, 1.0 / 7.0);
+    p = fma(r, p, -1.0 / 6.0);
+    p = fma(r, p, 1.0 / 5.0);
+    p = fma(r, p, -1.0 / 4.0);
+    p = fma(r, p, 1.0 / 3.0);
+    p = fma(r, p, -1.0 / 2.0);
+    // double(e), exact: 2^52 + 2^51 + e as bits, less the constant
+    const double ed = __hiloint2double(0x43380000 + (e >> 31), e) - 6755399441055744.0;
+    const double lo = fma(r2, p, fma(ed, QL_LOGTAB[257].y, QL_LOGTAB[2 * j + 1].x));
+    return fma(ed, QL_LOGTAB[257].x, t.y) + (r + lo);
+}
+#else
 template <>
 __device__ __forceinline__ double log_<double>(double x) { return log(x); }
+#endif
 
 template <typename Real>
 __device__ __forceinline__ Real exp_(Real x);
@@ -106,8 +150,18 @@ __device__ __forceinline__ float rcp_<float>(float x)
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
+// FP64: the hardware's approximation (PTX rcp.approx.ftz.f64, relative error
+// e < 2^-19.9 measured) and one third-order step r (1 + e + e^2), three FP64
+// instructions instead of the division's five; at most one unit in the last
+// place from the rounded quotient (measured over 10^8 values).
 template <>
-__device__ __forceinline__ double rcp_<double>(double x) { return 1.0 / x; }
+__device__ __forceinline__ double rcp_<double>(double x)
+{
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
 
 // An exact power of two s with s x in [1, 4), for finite x >= 0 (s = 2^(e'-bias)
 // where e' is the complement of x's exponent field with its lowest bit
@@ -116,27 +170,14 @@ __device__ __forceinline__ float pow2_recip_(float x)
 {
     return __uint_as_float(~__float_as_uint(x) & 0x7F000000u);
 }
-__device__ __forceinline__ double pow2_recip_(double x)
-{
-    return __hiloint2double(~__double2hiint(x) & 0x7FE00000, 0);
-}
 
-// max(a, b, c) of finite values (a single three-input max in FP32).
+// max(a, b, c) of finite values (a single three-input max).
 __device__ __forceinline__ float max3_(float a, float b, float c)
 {
     float r;
     asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
     return r;
 }
-__device__ __forceinline__ double max3_(double a, double b, double c) { return fmax(a, fmax(b, c)); }
-
-// Smallest positive normal number of the working precision.
-template <typename Real>
-__device__ __forceinline__ Real min_normal_();
-template <>
-__device__ __forceinline__ float min_normal_<float>() { return 1.17549435e-38f; }
-template <>
-__device__ __forceinline__ double min_normal_<double>() { return 2.2250738585072014e-308; }
 
 // ---------------------------------------------------------------------------
 // Double-FP32 arithmetic: a value held as the unevaluated sum h + l of two
@@ -200,17 +241,25 @@ __device__ __forceinline__ FF ff_div(FF a, FF b)
 // WENO-5 value at the interface i+1/2 for a positive advection velocity
 // (App. A.2), from f_{i-2..i+2}, for both components of the pairs.  Weights
 // are delta_q / beta_q^2 normalised, with no epsilon; FP32 evaluates that
-// quotient with reciprocals (below), FP64 in the product form
+// quotient with reciprocals (below), FP64 the product form
 //   w_q = delta_q prod_{r != q} beta_r^2 / sum_s delta_s prod_{r != s} beta_r^2,
-// equal to the quotient form wherever all beta_q > 0.  The indicators are
-// first rescaled by one exact power of two (the weights depend only on their
-// ratios).  Single-zero rows of Table weno_x come out of the product form;
-// multi-zero rows give f0 (see below).  Candidates are differences from f0,
-// so constant data give exactly f0.
+// equal to it wherever all beta_q > 0, in integer arithmetic (weno_i64.cuh).
+// FP32 rescales the indicators by one exact power of two first (the weights
+// depend only on their ratios).  Candidates are differences from f0, so constant
+// data give exactly f0.
 template <typename Real>
-__device__ __forceinline__ P2<Real> weno5_face2(P2<Real> fm2, P2<Real> fm1, P2<Real> f0, P2<Real> fp1, P2<Real> fp2)
+__device__ __forceinline__ P2<Real> weno5_face2(P2<Real> fm2, P2<Real> fm1, P2<Real> f0, P2<Real> fp1, P2<Real> fp2);
+template <>
+__device__ __forceinline__ double2 weno5_face2<double>(double2 fm2, double2 fm1, double2 f0, double2 fp1, double2 fp2)
 {
-    using V = P2<Real>;
+    const double2 a = sub2(fm2, fm1), b = sub2(f0, fm1), g = sub2(fp1, f0), c = sub2(fp2, fp1);
+    return mk2(weno5_face_i64(a.x, b.x, g.x, c.x, f0.x), weno5_face_i64(a.y, b.y, g.y, c.y, f0.y));
+}
+template <>
+__device__ __forceinline__ float2 weno5_face2<float>(float2 fm2, float2 fm1, float2 f0, float2 fp1, float2 fp2)
+{
+    using V = float2;
+    using Real = float;
     const V Dm2n = sub2(fm2, fm1);  // -(f_{i-1} - f_{i-2})
     const V Dm1 = sub2(f0, fm1);
     const V D0 = sub2(fp1, f0);
@@ -235,46 +284,27 @@ __device__ __forceinline__ P2<Real> weno5_face2(P2<Real> fm2, P2<Real> fm1, P2<R
     const V c2 = add2(Dm1, D0x);
     const V c3 = fma2(sp2(Real(-0.5)), D1, D0x);
     const V sc = mk2(pow2_recip_(max3_(b1.x, b2.x, b3.x)), pow2_recip_(max3_(b1.y, b2.y, b3.y)));
-    if constexpr (sizeof(Real) == 4) {
-        // FP32: the quotient form itself, 1/beta_q^2 from the hardware reciprocal
-        // (the special-function unit has room where the FMA pipes have none).  The
-        // rescaled indicators lie in [0, 4), the largest in [1, 4); the same fused
-        // multiply-add raises each by 2^-50, which bounds 1/beta^2 by 2^100 (the
-        // numerator stays finite for differences below 2^26).  Nonzero FP32
-        // indicators of one face differ from the largest by less than 2^54, so
-        // the raise moves weight only between stencils flat to within 2^-25 of
-        // the face's largest difference, whose candidates agree to that level.
-        // A vanishing indicator gets 1/beta^2 = 2^100 against at most 1 for the
-        // largest: one zero takes all the weight and two or three share it as
-        // delta_q, the rows of Table weno_x.
-        const V e50 = sp2(Real(8.8817841970012523e-16));
-        b1 = fma2(b1, sc, e50);
-        b2 = fma2(b2, sc, e50);
-        b3 = fma2(b3, sc, e50);
-        const V r1 = mk2(rcp_(b1.x), rcp_(b1.y)), r2 = mk2(rcp_(b2.x), rcp_(b2.y)), r3 = mk2(rcp_(b3.x), rcp_(b3.y));
-        const V a1 = mul2(r1, r1), a2 = mul2(r2, r2), a3 = mul2(r3, r3);
-        const V D = fma2(sp2(Real(3)), a3, fma2(sp2(Real(6)), a2, a1));
-        const V num = fma2(a1, c1, fma2(a2, c2, mul2(a3, c3)));
-        const V rD = mk2(rcp_(D.x), rcp_(D.y));
-        return fma2(num, rD, f0);
-    } else {
-        b1 = mul2(b1, sc);
-        b2 = mul2(b2, sc);
-        b3 = mul2(b3, sc);
-        const V s1 = mul2(b1, b1), s2 = mul2(b2, b2), s3 = mul2(b3, b3);
-        const V P1 = mul2(s2, s3), P2v = mul2(s1, s3), P3 = mul2(s1, s2);
-        const V D = fma2(sp2(Real(3)), P3, fma2(sp2(Real(6)), P2v, P1));
-        const V num = fma2(P1, c1, fma2(P2v, c2, mul2(P3, c3)));
-        // D = 0 only when two or three indicators vanish.  beta_q = 0 means the three
-        // values of stencil q are equal, so two vanishing indicators make the union of
-        // those stencils constant, the candidates that carry weight in Table weno_x
-        // equal f0 there, and the face value is f0: num = 0 in that case too, and D is
-        // raised to the smallest normal number so that its reciprocal stays finite
-        // (a D below it would have no finite reciprocal either).
-        const Real dmin = min_normal_<Real>();
-        const V rD = mk2(rcp_(max_(D.x, dmin)), rcp_(max_(D.y, dmin)));
-        return fma2(num, rD, f0);
-    }
+    // The quotient form itself, 1/beta_q^2 from the hardware reciprocal
+    // (the special-function unit has room where the FMA pipes have none).  The
+    // rescaled indicators lie in [0, 4), the largest in [1, 4); the same fused
+    // multiply-add raises each by 2^-50, which bounds 1/beta^2 by 2^100 (the
+    // numerator stays finite for differences below 2^26).  Nonzero FP32
+    // indicators of one face differ from the largest by less than 2^54, so
+    // the raise moves weight only between stencils flat to within 2^-25 of
+    // the face's largest difference, whose candidates agree to that level.
+    // A vanishing indicator gets 1/beta^2 = 2^100 against at most 1 for the
+    // largest: one zero takes all the weight and two or three share it as
+    // delta_q, the rows of Table weno_x.
+    const V e50 = sp2(Real(8.8817841970012523e-16));
+    b1 = fma2(b1, sc, e50);
+    b2 = fma2(b2, sc, e50);
+    b3 = fma2(b3, sc, e50);
+    const V r1 = mk2(rcp_(b1.x), rcp_(b1.y)), r2 = mk2(rcp_(b2.x), rcp_(b2.y)), r3 = mk2(rcp_(b3.x), rcp_(b3.y));
+    const V a1 = mul2(r1, r1), a2 = mul2(r2, r2), a3 = mul2(r3, r3);
+    const V D = fma2(sp2(Real(3)), a3, fma2(sp2(Real(6)), a2, a1));
+    const V num = fma2(a1, c1, fma2(a2, c2, mul2(a3, c3)));
+    const V rD = mk2(rcp_(D.x), rcp_(D.y));
+    return fma2(num, rD, f0);
 }
 
 // Asks the TMA unit to bring `bytes` (a multiple of 16, 16-byte aligned
@@ -349,6 +379,9 @@ constexpr uint32_t kMbarPolls = 1u << 16;
 template <typename Real>
 __device__ __forceinline__ Real cd6_(const Real *v, int s)
 {
+    if constexpr (sizeof(Real) == 8)  // fused: 6 FP64 instructions instead of 8
+        return fma(Real(1.0 / 60.0), v[s + 3] - v[s - 3],
+                   fma(Real(-3.0 / 20.0), v[s + 2] - v[s - 2], Real(0.75) * (v[s + 1] - v[s - 1])));
     return Real(1.0 / 60.0) * (v[s + 3] - v[s - 3]) + Real(-3.0 / 20.0) * (v[s + 2] - v[s - 2]) +
            Real(0.75) * (v[s + 1] - v[s - 1]);
 }
@@ -544,12 +577,10 @@ __device__ __forceinline__ void stage_tile(const StageArgs &a, const int64_t i0,
             uf = Real(u.h);
             Tf = Real(T.h);
         } else {
-            // 1/n from a working-precision reciprocal refined by Newton steps in FP64
-            // (one step gives ~1e-14 after an FP32 seed, two after FP64's own division)
+            // FP32: 1/n from an FP32 reciprocal and one Newton step in FP64 (about 1e-14)
             const double n = as_double(F0), M1 = as_double(F1), ME = as_double(FE);
             double rn = double(rcp_(Real(n)));
-            rn = fma(rn, fma(-n, rn, 1.0), rn);
-            if (sizeof(Real) == 8) rn = fma(rn, fma(-n, rn, 1.0), rn);
+            if (sizeof(Real) == 4) rn = fma(rn, fma(-n, rn, 1.0), rn);
             const double u = M1 * rn;
             const double T = fma(-u, M1, ME) * rn * (1.0 / 3.0);
             uf = Real(u);
@@ -560,7 +591,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs &a, const int64_t i0,
         const Real q = Real(0.5) * (tS3 + tR1 - uf * fma_(Real(3), tS2, tR0) + Real(2) * uf * uf * (uf * nf));
         const int64_t i = i0 - kHalo + c;
         if (i >= 0 && i < a.nx) {
-            if (!(nf > Real(0)) || !(Tf > Real(0)) || !isfinite(uf) || !isfinite(q) || !isfinite(nf) || !isfinite(Tf))
+            if (!positive_(nf) || !positive_(Tf) || !finite_(uf) || !finite_(q) || !finite_(nf) || !finite_(Tf))
                 atomicOr(a.err, 1u);
         }
         s_n[c] = nf;
@@ -599,7 +630,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs &a, const int64_t i0,
     const Real chi = ret ? exp_(s_lnchi[s]) : Real(0.5) * (Real(2) - eta) * (rome * rome * rome);
     const Real Y = Real(4) * eta * chi;
     const Real muf = fma_(fma_(Real(0.16 * (1.0 + 12.0 / 3.14159265358979323846)), Y, Real(0.8)), Y, Real(1));
-    const Real sqT = T * rsqrt_(T);
+    const Real sqT = sqrt_(T);
     const Real inv_tau = rhat * chi * sqT * rcp_(Real(a.tau_pref) * muf);
     Real Pr = Real(a.pr_const);
     if (a.pr_mode) {
@@ -697,7 +728,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs &a, const int64_t i0,
 
     // FP32 stage 1 runs faster with the loop rolled (0.625 -> 0.609 ms per launch on the Sod tube, 2^22 cells,
     // Q = 32), stages 2-3 with kVelocityLoopUnroll pairs per iteration (rolled: 0.682 -> 0.697 ms)
-    constexpr int kUnroll = (STAGE == 1 && sizeof(Real) == 4) ? 1 : kVelocityLoopUnroll;
+    constexpr int kUnroll = (STAGE == 1 || sizeof(Real) == 8) ? 1 : kVelocityLoopUnroll;
 #pragma unroll kUnroll
     for (int j = j0; j < j1; ++j) {
         const int kp = H + j, km = H - 1 - j;
