@@ -61,7 +61,8 @@ __global__ void fdlb_periodic_ghost_kernel(P2<Real> *__restrict__ psi, int64_t n
 
 // ---------------------------------------------------------------------------
 // chi_RET-FM.  Density sum_k phi_k of every interior cell of a state, in the
-// order of the stage kernel's output sum (pairs k = H + j, H - 1 - j).
+// order of the stage kernel's output sum (pairs k = H + j, H - 1 - j; FP64 sums
+// groups of pairs, as its moments).
 template <typename Real, int Q>
 __global__ void fdlb_density_kernel(const P2<Real> *__restrict__ psi, int64_t nx, int64_t stride,
                                     Real *__restrict__ n)
@@ -69,9 +70,14 @@ __global__ void fdlb_density_kernel(const P2<Real> *__restrict__ psi, int64_t nx
     constexpr int H = Q / 2;
     const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= nx) return;
+    constexpr int GRP = sizeof(Real) == 8 ? SumGroup<Real>::pairs : H;
     Real acc = Real(0);
-    for (int j = 0; j < H; ++j)
-        acc += psi[int64_t(H + j) * stride + kHalo + i].x + psi[int64_t(H - 1 - j) * stride + kHalo + i].x;
+    for (int g = 0; g < H; g += GRP) {
+        Real part = Real(0);
+        for (int j = g; j < g + GRP && j < H; ++j)
+            part += psi[int64_t(H + j) * stride + kHalo + i].x + psi[int64_t(H - 1 - j) * stride + kHalo + i].x;
+        acc += part;
+    }
     n[i] = acc;
 }
 

@@ -11,4 +11,5 @@ static __device__ double2 QL_LOGTAB[258];
 #define QL_REAL double
 #define QL_SUFFIX f64
 #include "fdlb_impl.cuh"
+#include "fdlb_cells.cuh"
 #include "fdlb_lq.cuh"

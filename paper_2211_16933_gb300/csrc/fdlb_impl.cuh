@@ -57,39 +57,48 @@ cudaError_t QL_FN(upload_tables_)(const double *all)
     return cudaMemcpyToSymbol(QL_TAB, host, sizeof(host));
 }
 
-// One CTA per tile; in FP64, a domain of fewer tiles than the GPU holds CTAs
-// splits each tile's velocity pairs over up to Q/2 CTAs (FP64 arithmetic, not
-// memory, bounds those small domains).  With chi_RET-FM the densities of the
+// One CTA per tile; in FP64, a domain of fewer tiles than the GPU has SMs splits
+// each tile's velocity pairs over up to Q/2 CTAs (FP64 arithmetic, not memory,
+// bounds those small domains).  The split with the least FP64 instructions per
+// thread on the busiest SM is taken: about 8 Q + 170 for the per-cell part, which
+// every CTA of a tile repeats, and Q + 52 per velocity pair.  With chi_RET-FM the densities of the
 // output then come from a separate pass, in the order the stage sums them.
 template <int Q, int STAGE, bool RET>
 static cudaError_t stage_q(const StageArgs &a, cudaStream_t s)
 {
-    constexpr size_t smem = stage_smem_bytes<QL_REAL, Q, kWarps, RET>();
+    constexpr int W = stage_warps<QL_REAL>();
+    constexpr size_t smem = stage_smem_bytes<QL_REAL, Q, W, RET>();
     auto kern = fdlb_stage_kernel<QL_REAL, Q, STAGE, RET>;
-    static int resident[64] = {};  // CTAs of this kernel the device holds at once
+    static int sm_count[64] = {};
     int dev = 0;
     cudaGetDevice(&dev);
-    if (!resident[dev & 63]) {
+    if (!sm_count[dev & 63]) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-        int per_sm = 0, sms = 0;
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem);
+        int sms = 0;
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return e;
-        resident[dev & 63] = per_sm * sms > 0 ? per_sm * sms : 1;
+        sm_count[dev & 63] = sms > 0 ? sms : 1;
     }
-    const int64_t nt = num_tiles(a.nx);
+    const int64_t nt = (a.nx + TileShape<W>::tile - 1) / TileShape<W>::tile;
     StageArgs b = a;
     b.vsplit = 1;
-    if (sizeof(QL_REAL) == 8 && nt < resident[dev & 63]) {
-        const int64_t v = resident[dev & 63] / nt;
-        b.vsplit = int(v < Q / 2 ? v : Q / 2);
+    const int sms = sm_count[dev & 63];
+    if (sizeof(QL_REAL) == 8 && nt < sms) {
+        int64_t best = 0;
+        for (int v = 1; v <= Q / 2; ++v) {
+            const int64_t cost = (nt * v + sms - 1) / sms * (8 * Q + 170 + (Q + 52) * ((Q / 2 + v - 1) / v));
+            if (v == 1 || cost < best) {
+                best = cost;
+                b.vsplit = v;
+            }
+        }
     }
     // programmatic stream serialisation: the launch may overlap the tail of the
     // previous kernel in the stream, which the kernel waits for before its
     // first access to memory
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(unsigned(nt * b.vsplit));
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(32 * W);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute at[1];

@@ -386,6 +386,201 @@ __device__ __forceinline__ Real cd6_(const Real *v, int s)
            Real(0.75) * (v[s + 1] - v[s - 1]);
 }
 
+// ---------------------------------------------------------------------------
+// Per-cell pieces of the right-hand side, shared by the tile kernels below and the
+// kernels of small domains (fdlb_cells.cuh), which must give the same bits.
+
+// Raw moment sums (Sec. II.D) of a group of velocity pairs: (S0, R0), (S1, R1),
+// S2, S3 with S_j = sum p^j phi and R_j = sum p^j theta.
+template <typename Real>
+struct GroupSums {
+    P2<Real> s01, s11;
+    Real s2, s3;
+    __device__ __forceinline__ GroupSums() : s01(sp2(Real(0))), s11(sp2(Real(0))), s2(Real(0)), s3(Real(0)) {}
+    // the pair of velocities p (state fa) and -p (fb)
+    __device__ __forceinline__ void add(Real p, Real p2, Real p3, P2<Real> fa, P2<Real> fb)
+    {
+        const P2<Real> sm = add2(fa, fb), df = sub2(fa, fb);
+        s01 = add2(s01, sm);
+        s11 = fma2(sp2(p), df, s11);
+        s2 = fma_(p2, sm.x, s2);
+        s3 = fma_(p3, df.x, s3);
+    }
+};
+// Velocity pairs per group: 8 in FP32 (a group's FP32 sums are combined in higher
+// precision); 4 in FP64, so that the small-domain kernels can sum groups in parallel.
+template <typename Real>
+struct SumGroup {
+    static constexpr int pairs = sizeof(Real) == 8 ? 4 : 8;
+};
+
+// The groups' sums combined in group order, then n, u, T and q.  FP64 mode sums
+// in FP64.  FP32 mode combines the groups' mass, momentum and energy sums
+// either in double-FP32 (FF) or in FP64 (a.sums64), deriving u and T in the same
+// arithmetic (FP64 runs at a small fraction of the FP32 rate on this GPU); the
+// heat-flux sums stay in FP32.
+template <typename Real>
+struct MomentSums {
+    // the FP64 sums share the registers of the double-FP32 ones: a double is held
+    // as its two 32-bit halves in (h, l)
+    FF F0{0.f, 0.f}, F1{0.f, 0.f}, FE{0.f, 0.f};
+    Real tS2 = 0, tS3 = 0, tR0 = 0, tR1 = 0;
+    __device__ __forceinline__ void add(const GroupSums<Real> &g, bool ff)
+    {
+        if (ff) {
+            // error-free accumulation: h takes the rounded sum, l its errors
+            const FF a0 = two_sum(F0.h, float(g.s01.x)), a1 = two_sum(F1.h, float(g.s11.x));
+            const FF a2 = two_sum(FE.h, float(g.s2)), a3 = two_sum(a2.h, float(g.s01.y));
+            F0 = {a0.h, F0.l + a0.l};
+            F1 = {a1.h, F1.l + a1.l};
+            FE = {a3.h, FE.l + (a2.l + a3.l)};
+        } else {
+            F0 = as_ff(as_double(F0) + double(g.s01.x));
+            F1 = as_ff(as_double(F1) + double(g.s11.x));
+            FE = as_ff(as_double(FE) + double(g.s2 + g.s01.y));
+        }
+        tS2 += g.s2;
+        tS3 += g.s3;
+        tR0 += g.s01.y;
+        tR1 += g.s11.y;
+    }
+    __device__ __forceinline__ void finish(bool ff, Real &nf, Real &uf, Real &Tf, Real &q) const
+    {
+        // 3 n T = sum xi^2 phi + sum theta = (S2 + R0) - u S1
+        if (ff) {
+            const FF n = fast_two_sum(F0.h, F0.l), m1 = fast_two_sum(F1.h, F1.l), me = fast_two_sum(FE.h, FE.l);
+            const FF u = ff_div(m1, n);
+            const FF T = ff_div(ff_add(me, ff_neg(ff_mul(u, m1))), ff_mul_f(n, 3.0f));
+            nf = Real(n.h);
+            uf = Real(u.h);
+            Tf = Real(T.h);
+        } else {
+            // FP32: 1/n from an FP32 reciprocal and one Newton step in FP64 (about 1e-14)
+            const double n = as_double(F0), M1 = as_double(F1), ME = as_double(FE);
+            double rn = double(rcp_(Real(n)));
+            if (sizeof(Real) == 4) rn = fma(rn, fma(-n, rn, 1.0), rn);
+            const double u = M1 * rn;
+            const double T = fma(-u, M1, ME) * rn * (1.0 / 3.0);
+            uf = Real(u);
+            Tf = Real(T);
+            nf = Real(n);
+        }
+        // 2 q = sum xi^3 phi + sum xi theta = S3 + R1 - u (3 S2 + R0) + 2 u^2 S1
+        q = Real(0.5) * (tS3 + tR1 - uf * fma_(Real(3), tS2, tR0) + Real(2) * uf * uf * (uf * nf));
+    }
+};
+template <typename Real>
+__device__ __forceinline__ bool nonphysical_(Real n, Real u, Real T, Real q)
+{
+    return !positive_(n) || !positive_(T) || !finite_(u) || !finite_(q) || !finite_(n) || !finite_(T);
+}
+
+// Eq. (chi_ret): chi_SET of the averaged density nbar.
+template <typename Real>
+__device__ __forceinline__ Real chi_of_nbar_(const StageArgs &a, Real nbar)
+{
+    const Real eb = Real(a.eta0) * nbar * Real(a.inv_rho_ref), omb = Real(1) - eb;
+    return Real(0.5) * (Real(2) - eb) / (omb * omb * omb);
+}
+
+// Runge-Kutta weight of v = psi + dt L in a stage's output (c psi^n + w v): 1,
+// 1/4 and fl(2/3), whose complement 1 - w is exact (Sterbenz).
+template <typename Real>
+__device__ __forceinline__ Real rk_weight_(int stage)
+{
+    return stage == 2 ? Real(0.25) : (stage == 3 ? Real(2.0 / 3.0) : Real(1));
+}
+
+// Collision coefficients of a cell (Secs. II.A-II.C, Eq. j1_expanded): the targets
+// times n g_k as P(+-p) = E(p^2) +- p O(p^2), E = D0 + D2 p^2 and O = D1 + D3 p^2
+// (pairs for phi and theta, times 2 T for theta), and the factor kpsi of psi.
+template <typename Real>
+struct CellCoefs {
+    P2<Real> D0, D1, D2, D3;
+    Real kpsi;
+};
+// dlnn, du, dlnT: gradients; chi_RET-FM (RET): chi of the cell and the gradient
+// of ln chi (both unused otherwise).
+template <typename Real, bool RET>
+__device__ __forceinline__ CellCoefs<Real> cell_coefs_(const StageArgs &a, int stage, Real n, Real u, Real T, Real q,
+                                                       Real dlnn, Real du, Real dlnT, Real chi_ret, Real dlnchi_ret)
+{
+    using V = P2<Real>;
+    const Real rk_w = rk_weight_<Real>(stage);
+    // Secs. II.A-B: eta, chi_SET, Y = b rho chi, tau = mu / P_i, Pr.
+    const Real rhat = n * Real(a.inv_rho_ref);
+    const Real eta = Real(a.eta0) * rhat;
+    const Real ome = Real(1) - eta;
+    const Real rome = rcp_(ome);
+    const Real chi = RET ? chi_ret : Real(0.5) * (Real(2) - eta) * (rome * rome * rome);
+    const Real Y = Real(4) * eta * chi;
+    const Real muf = fma_(fma_(Real(0.16 * (1.0 + 12.0 / 3.14159265358979323846)), Y, Real(0.8)), Y, Real(1));
+    const Real sqT = sqrt_(T);
+    const Real inv_tau = rhat * chi * sqT * rcp_(Real(a.tau_pref) * muf);
+    Real Pr = Real(a.pr_const);
+    if (a.pr_mode) {
+        const Real laf =
+            fma_(fma_(Real(0.36 * (1.0 + 32.0 / (9.0 * 3.14159265358979323846))), Y, Real(1.2)), Y, Real(1));
+        Pr = Real(2.0 / 3.0) * muf * rcp_(laf);
+    }
+    const Real invT = rcp_(T);
+    // Shakhov: A = (1 - Pr) q / (5 P_i T), P_i = n T
+    const Real A = (Real(1) - Pr) * q * invT * invT * (Real(0.2) * rcp_(n));
+    const Real Yj = a.enskog ? Y : Real(0);
+    // chi_SET: d ln chi = eta (3/(1-eta) - 1/(2-eta)) d ln rho (chi depends on the local eta only);
+    // chi_RET-FM: 6th-order difference of ln chi(nbar)
+    const Real dlnchi = RET ? dlnchi_ret : eta * (Real(3) * rome - rcp_(Real(2) - eta)) * dlnn;
+    const Real G = dlnchi + Real(2) * dlnn;
+    // Targets over the equilibrium, cubic in xi = p_k - u:
+    //   phi:   (1/tau)(1 + A xi (xi^2/T - 3)) - Y [xi G + 3/5 (xi^2/T - 1) du + 3/10 (xi^3/T + xi/3) dlnT]
+    //   theta: (1/tau)(1 + A xi (xi^2/T - 1)) - Y [xi G + 3/5 (xi^2/T - 1/3) du + 3/10 (xi^3/T + 7 xi/3) dlnT]
+    // times n g_k and 2 T n g_k; the pairs below hold (phi, theta) coefficients
+    // already multiplied by n and 2 T n.
+    const Real a0 = fma_(Real(0.6) * Yj, du, inv_tau);
+    const Real a1 = -Real(3) * A * inv_tau - Yj * G - Real(0.1) * Yj * dlnT;
+    const Real a2 = -Real(0.6) * Yj * du * invT;
+    const Real a3 = (A * inv_tau - Real(0.3) * Yj * dlnT) * invT;
+    const Real b0 = fma_(Real(0.2) * Yj, du, inv_tau);
+    const Real b1 = -A * inv_tau - Yj * G - Real(0.7) * Yj * dlnT;
+    // Stages 1-3 fold dt and the Runge-Kutta weight of v into the targets (see
+    // the velocity loop).
+    const Real ndt = stage == 0 ? n : n * (Real(a.dt) * rk_w);
+    const Real nphi = ndt, nth = Real(2) * T * ndt;
+    const V C0 = mk2(a0 * nphi, b0 * nth), C1 = mk2(a1 * nphi, b1 * nth);
+    const V C2 = mk2(a2 * nphi, a2 * nth), C3 = mk2(a3 * nphi, a3 * nth);
+    // The same cubic as a polynomial in y = xi + u = +-p (Taylor shift by -u,
+    // Horner's scheme): P(+-p) = E(p^2) +- p O(p^2) with E = D0 + D2 p^2 and
+    // O = D1 + D3 p^2, so both velocities of a pair share E and O.
+    V D0 = C0, D1 = C1, D2 = C2;
+    const V D3 = C3;
+    {
+        const V mu = sp2(-u);
+        D2 = fma2(mu, D3, D2);
+        D1 = fma2(mu, D2, D1);
+        D0 = fma2(mu, D1, D0);
+        D2 = fma2(mu, D3, D2);
+        D1 = fma2(mu, D2, D1);
+        D2 = fma2(mu, D3, D2);
+    }
+    CellCoefs<Real> c;
+    c.D0 = D0;
+    c.D1 = D1;
+    c.D2 = D2;
+    c.D3 = D3;
+    // STAGE 0: L[psi] = target - psi / tau - advection.  Stages 1-3 form
+    // w v = w (psi + dt L[psi]) directly as w (1 - dt/tau) psi + w dt target -
+    // w dt advection (targets and the advection factor already scaled by w dt).
+    c.kpsi = stage == 0 ? -inv_tau : rk_w * (Real(1) - Real(a.dt) * inv_tau);
+    return c;
+}
+
+// Advection factor p adv of a velocity: w dt p / dx (p / dx for STAGE 0).
+template <typename Real>
+__device__ __forceinline__ Real advection_(const StageArgs &a, int stage)
+{
+    return stage == 0 ? Real(a.inv_dx) : Real(a.dt) * rk_weight_<Real>(stage) * Real(a.inv_dx);
+}
+
 // CTA shape: WARPS warps update 31 WARPS cells and stage 4 more on each side.
 template <int WARPS>
 struct TileShape {
@@ -394,7 +589,7 @@ struct TileShape {
     static constexpr int seg = tile + 2 * kHalo;
 };
 
-// Shared memory of one stage CTA: the staged rows, 6 per-cell arrays, 2 more
+// Shared memory of one stage CTA: the staged rows, 6 per-cell arrays, 3 more
 // for chi_RET-FM, and 3 pairs per velocity pair.  The equilibrium table rows
 // G[k][l] are read from the constant bank (every lane of a warp reads the same
 // entry), which leaves the shared memory to the staged rows.
@@ -402,7 +597,7 @@ template <typename Real, int Q, int WARPS, bool RET = false>
 constexpr size_t stage_smem_bytes()
 {
     constexpr int SEG = TileShape<WARPS>::seg;
-    return sizeof(P2<Real>) * size_t(Q) * SEG + sizeof(Real) * ((RET ? 8 : 6) * size_t(SEG)) +
+    return sizeof(P2<Real>) * size_t(Q) * SEG + sizeof(Real) * ((RET ? 9 : 6) * size_t(SEG)) +
            sizeof(P2<Real>) * 3 * size_t(Q / 2);
 }
 
@@ -455,13 +650,12 @@ __device__ __forceinline__ void stage_tile(const StageArgs &a, const int64_t i0,
     Real *s_lnn = s_q + SEG;
     Real *s_lnT = s_lnn + SEG;
     Real *s_lnchi = s_lnT + SEG;  // chi_RET-FM: nbar, then ln chi(nbar)
-    Real *s_nout = s_lnchi + SEG; // chi_RET-FM: density of the output, per owned cell
+    Real *s_chi = s_lnchi + SEG;  // chi_RET-FM: chi(nbar)
+    Real *s_nout = s_chi + SEG;   // chi_RET-FM: density of the output, per owned cell
     // per velocity pair j: (p, p), (p^2, p^2), (w dt p / dx, w dt p / dx)
-    V *s_pt = reinterpret_cast<V *>(s_n + SEG * (RET ? 8 : 6));
+    V *s_pt = reinterpret_cast<V *>(s_n + SEG * (RET ? 9 : 6));
     constexpr bool ret = RET;  // chi_RET-FM: a.nbar and a.nout are set
-    // Runge-Kutta weight of v = psi + dt L in the stage output (c psi^n + w v):
-    // 1, 1/4 and fl(2/3), whose complement 1 - w is exact (Sterbenz)
-    const Real rk_w = STAGE == 2 ? Real(0.25) : (STAGE == 3 ? Real(2.0 / 3.0) : Real(1));
+    const Real rk_w = rk_weight_<Real>(STAGE);
 
     const int t = threadIdx.x;
     const int64_t stride = a.stride;
@@ -496,7 +690,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs &a, const int64_t i0,
         }
         if (t < H) {
             const Real p = QL_TAB[TV.p + H + t];
-            const Real adv = STAGE == 0 ? Real(a.inv_dx) : Real(a.dt) * rk_w * Real(a.inv_dx);
+            const Real adv = advection_<Real>(a, STAGE);
             s_pt[3 * t] = sp2(p);
             s_pt[3 * t + 1] = sp2(QL_TAB[TV.p2 + H + t]);
             s_pt[3 * t + 2] = sp2(p * adv);
@@ -523,77 +717,24 @@ __device__ __forceinline__ void stage_tile(const StageArgs &a, const int64_t i0,
         __syncthreads();
     }
 
-    // 2. Moments of staged cell c (cell i0 - kHalo + c), Sec. II.D, from raw
-    //    sums over velocity pairs.  FP64 mode sums in FP64.  FP32 mode sums
-    //    groups of 8 pairs in FP32 and combines the groups' mass, momentum and
-    //    energy sums either in FP64 (a.sums64) or in double-FP32 arithmetic,
-    //    deriving u and T in the same arithmetic (FP64 runs at a small fraction
-    //    of the FP32 rate on this GPU); the heat-flux sums stay in FP32.
+    // 2. Moments of staged cell c (cell i0 - kHalo + c), Sec. II.D.
     const bool kFF = sizeof(Real) == 4 && !QL_F32_SUMS_FP64 && !a.sums64;
     for (int c = t; c < SEG; c += THREADS) {
-        constexpr int GRP = sizeof(Real) == 8 ? H : 8;
-        // the FP64 sums (FP64 mode, or a.sums64) share the registers of the
-        // double-FP32 ones: a double is held as its two 32-bit halves in (h, l)
-        FF F0{0.f, 0.f}, F1{0.f, 0.f}, FE{0.f, 0.f};
-        Real tS2 = 0, tS3 = 0, tR0 = 0, tR1 = 0;
+        constexpr int GRP = SumGroup<Real>::pairs;
+        MomentSums<Real> ms;
 #pragma unroll
         for (int g = 0; g < H; g += GRP) {
-            V s01 = sp2(Real(0)), s11 = sp2(Real(0));  // (S0, R0), (S1, R1) partials
-            Real s2 = 0, s3 = 0;
+            GroupSums<Real> gs;
 #pragma unroll
-            for (int j = g; j < g + GRP && j < H; ++j) {
-                const Real p = QL_TAB[TV.p + H + j];
-                const V fa = s_psi[(H + j) * SEG + c], fb = s_psi[(H - 1 - j) * SEG + c];
-                const V sm = add2(fa, fb), df = sub2(fa, fb);
-                s01 = add2(s01, sm);
-                s11 = fma2(sp2(p), df, s11);
-                s2 = fma_(QL_TAB[TV.p2 + H + j], sm.x, s2);
-                s3 = fma_(QL_TAB[TV.p3 + H + j], df.x, s3);
-            }
-            if (kFF) {
-                // error-free accumulation: h takes the rounded sum, l its errors
-                const FF a0 = two_sum(F0.h, float(s01.x)), a1 = two_sum(F1.h, float(s11.x));
-                const FF a2 = two_sum(FE.h, float(s2)), a3 = two_sum(a2.h, float(s01.y));
-                F0 = {a0.h, F0.l + a0.l};
-                F1 = {a1.h, F1.l + a1.l};
-                FE = {a3.h, FE.l + (a2.l + a3.l)};
-            } else {
-                F0 = as_ff(as_double(F0) + double(s01.x));
-                F1 = as_ff(as_double(F1) + double(s11.x));
-                FE = as_ff(as_double(FE) + double(s2 + s01.y));
-            }
-            tS2 += s2;
-            tS3 += s3;
-            tR0 += s01.y;
-            tR1 += s11.y;
+            for (int j = g; j < g + GRP && j < H; ++j)
+                gs.add(QL_TAB[TV.p + H + j], QL_TAB[TV.p2 + H + j], QL_TAB[TV.p3 + H + j], s_psi[(H + j) * SEG + c],
+                       s_psi[(H - 1 - j) * SEG + c]);
+            ms.add(gs, kFF);
         }
-        // 3 n T = sum xi^2 phi + sum theta = (S2 + R0) - u S1
-        Real uf, Tf, nf;
-        if (kFF) {
-            const FF n = fast_two_sum(F0.h, F0.l), m1 = fast_two_sum(F1.h, F1.l), me = fast_two_sum(FE.h, FE.l);
-            const FF u = ff_div(m1, n);
-            const FF T = ff_div(ff_add(me, ff_neg(ff_mul(u, m1))), ff_mul_f(n, 3.0f));
-            nf = Real(n.h);
-            uf = Real(u.h);
-            Tf = Real(T.h);
-        } else {
-            // FP32: 1/n from an FP32 reciprocal and one Newton step in FP64 (about 1e-14)
-            const double n = as_double(F0), M1 = as_double(F1), ME = as_double(FE);
-            double rn = double(rcp_(Real(n)));
-            if (sizeof(Real) == 4) rn = fma(rn, fma(-n, rn, 1.0), rn);
-            const double u = M1 * rn;
-            const double T = fma(-u, M1, ME) * rn * (1.0 / 3.0);
-            uf = Real(u);
-            Tf = Real(T);
-            nf = Real(n);
-        }
-        // 2 q = sum xi^3 phi + sum xi theta = S3 + R1 - u (3 S2 + R0) + 2 u^2 S1
-        const Real q = Real(0.5) * (tS3 + tR1 - uf * fma_(Real(3), tS2, tR0) + Real(2) * uf * uf * (uf * nf));
+        Real nf, uf, Tf, q;
+        ms.finish(kFF, nf, uf, Tf, q);
         const int64_t i = i0 - kHalo + c;
-        if (i >= 0 && i < a.nx) {
-            if (!positive_(nf) || !positive_(Tf) || !finite_(uf) || !finite_(q) || !finite_(nf) || !finite_(Tf))
-                atomicOr(a.err, 1u);
-        }
+        if (i >= 0 && i < a.nx && nonphysical_(nf, uf, Tf, q)) atomicOr(a.err, 1u);
         s_n[c] = nf;
         s_u[c] = uf;
         s_T[c] = Tf;
@@ -601,9 +742,9 @@ __device__ __forceinline__ void stage_tile(const StageArgs &a, const int64_t i0,
         s_lnn[c] = log_(nf);
         s_lnT[c] = log_(Tf);
         if (ret) {
-            // Eq. (chi_ret): chi_SET of the averaged density
-            const Real eb = Real(a.eta0) * s_lnchi[c] * Real(a.inv_rho_ref), omb = Real(1) - eb;
-            s_lnchi[c] = log_(Real(0.5) * (Real(2) - eb) / (omb * omb * omb));
+            const Real chi = chi_of_nbar_(a, s_lnchi[c]);
+            s_chi[c] = chi;
+            s_lnchi[c] = log_(chi);
         }
     }
     __syncthreads();
@@ -622,62 +763,9 @@ __device__ __forceinline__ void stage_tile(const StageArgs &a, const int64_t i0,
     const Real du = cd6_(s_u, s) * inv_dx;
     const Real dlnT = cd6_(s_lnT, s) * inv_dx;
 
-    // Secs. II.A-B: eta, chi_SET, Y = b rho chi, tau = mu / P_i, Pr.
-    const Real rhat = n * Real(a.inv_rho_ref);
-    const Real eta = Real(a.eta0) * rhat;
-    const Real ome = Real(1) - eta;
-    const Real rome = rcp_(ome);
-    const Real chi = ret ? exp_(s_lnchi[s]) : Real(0.5) * (Real(2) - eta) * (rome * rome * rome);
-    const Real Y = Real(4) * eta * chi;
-    const Real muf = fma_(fma_(Real(0.16 * (1.0 + 12.0 / 3.14159265358979323846)), Y, Real(0.8)), Y, Real(1));
-    const Real sqT = sqrt_(T);
-    const Real inv_tau = rhat * chi * sqT * rcp_(Real(a.tau_pref) * muf);
-    Real Pr = Real(a.pr_const);
-    if (a.pr_mode) {
-        const Real laf =
-            fma_(fma_(Real(0.36 * (1.0 + 32.0 / (9.0 * 3.14159265358979323846))), Y, Real(1.2)), Y, Real(1));
-        Pr = Real(2.0 / 3.0) * muf * rcp_(laf);
-    }
-    const Real invT = rcp_(T);
-    // Shakhov: A = (1 - Pr) q / (5 P_i T), P_i = n T
-    const Real A = (Real(1) - Pr) * q * invT * invT * (Real(0.2) * rcp_(n));
-    const Real Yj = a.enskog ? Y : Real(0);
-    // chi_SET: d ln chi = eta (3/(1-eta) - 1/(2-eta)) d ln rho (chi depends on the local eta only);
-    // chi_RET-FM: 6th-order difference of ln chi(nbar)
-    const Real dlnchi =
-        ret ? cd6_(s_lnchi, s) * inv_dx : eta * (Real(3) * rome - rcp_(Real(2) - eta)) * dlnn;
-    const Real G = dlnchi + Real(2) * dlnn;
-    // Targets over the equilibrium, cubic in xi = p_k - u:
-    //   phi:   (1/tau)(1 + A xi (xi^2/T - 3)) - Y [xi G + 3/5 (xi^2/T - 1) du + 3/10 (xi^3/T + xi/3) dlnT]
-    //   theta: (1/tau)(1 + A xi (xi^2/T - 1)) - Y [xi G + 3/5 (xi^2/T - 1/3) du + 3/10 (xi^3/T + 7 xi/3) dlnT]
-    // times n g_k and 2 T n g_k; the pairs below hold (phi, theta) coefficients
-    // already multiplied by n and 2 T n.
-    const Real a0 = fma_(Real(0.6) * Yj, du, inv_tau);
-    const Real a1 = -Real(3) * A * inv_tau - Yj * G - Real(0.1) * Yj * dlnT;
-    const Real a2 = -Real(0.6) * Yj * du * invT;
-    const Real a3 = (A * inv_tau - Real(0.3) * Yj * dlnT) * invT;
-    const Real b0 = fma_(Real(0.2) * Yj, du, inv_tau);
-    const Real b1 = -A * inv_tau - Yj * G - Real(0.7) * Yj * dlnT;
-    // Stages 1-3 fold dt and the Runge-Kutta weight of v into the targets (see
-    // the velocity loop).
-    const Real ndt = STAGE == 0 ? n : n * (Real(a.dt) * rk_w);
-    const Real nphi = ndt, nth = Real(2) * T * ndt;
-    const V C0 = mk2(a0 * nphi, b0 * nth), C1 = mk2(a1 * nphi, b1 * nth);
-    const V C2 = mk2(a2 * nphi, a2 * nth), C3 = mk2(a3 * nphi, a3 * nth);
-    // The same cubic as a polynomial in y = xi + u = +-p (Taylor shift by -u,
-    // Horner's scheme): P(+-p) = E(p^2) +- p O(p^2) with E = D0 + D2 p^2 and
-    // O = D1 + D3 p^2, so both velocities of a pair share E and O.
-    V D0 = C0, D1 = C1, D2 = C2;
-    const V D3 = C3;
-    {
-        const V mu = sp2(-u);
-        D2 = fma2(mu, D3, D2);
-        D1 = fma2(mu, D2, D1);
-        D0 = fma2(mu, D1, D0);
-        D2 = fma2(mu, D3, D2);
-        D1 = fma2(mu, D2, D1);
-        D2 = fma2(mu, D3, D2);
-    }
+    const CellCoefs<Real> cc = cell_coefs_<Real, RET>(a, STAGE, n, u, T, q, dlnn, du, dlnT, ret ? s_chi[s] : Real(0),
+                                                      ret ? cd6_(s_lnchi, s) * inv_dx : Real(0));
+    const V D0 = cc.D0, D1 = cc.D1, D2 = cc.D2, D3 = cc.D3, kpsi = sp2(cc.kpsi);
 
     // Hermite coefficients of the equilibrium, Eq. (g_alpha), scaled as
     // d_l = l! c_l: d_0 = 1, d_1 = u, d_l = u d_{l-1} + (l-1)(T-1) d_{l-2} (the
@@ -698,11 +786,6 @@ __device__ __forceinline__ void stage_tile(const StageArgs &a, const int64_t i0,
         }
     }
 
-    // STAGE 0: L[psi] = target - psi / tau - advection.  Stages 1-3 form
-    // w v = w (psi + dt L[psi]) directly as w (1 - dt/tau) psi + w dt target -
-    // w dt advection (targets and the advection table already scaled by w dt).
-    const Real dt = Real(a.dt);
-    const V kpsi = sp2(STAGE == 0 ? -inv_tau : rk_w * (Real(1) - dt * inv_tau));
     const V *__restrict__ base = static_cast<const V *>(a.base);
     V *out = static_cast<V *>(a.out);
     const int64_t col = kHalo + i;
@@ -714,6 +797,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs &a, const int64_t i0,
     // velocities leaves it to a density pass after the stage
     const bool own_density = RET && STAGE != 0 && (sizeof(Real) == 4 || nparts == 1);
     if (own_density && owner) s_nout[s] = Real(0);
+    Real dens = Real(0);
 
     // psi^n rows of the tile's cells (columns kHalo + i0 .. kHalo + i0 + tile - 1,
     // inside every row, whose stride leaves room for the staged segment): before
@@ -781,7 +865,17 @@ __device__ __forceinline__ void stage_tile(const StageArgs &a, const int64_t i0,
             // streaming stores: the next stage reads them from memory, not from L2
             __stcs(out + ip, op);
             __stcs(out + im, om);
-            if (own_density) s_nout[s] += op.x + om.x;
+            if (own_density) {
+                if (sizeof(Real) == 8) {  // in the groups of the moments
+                    dens += op.x + om.x;
+                    if ((j + 1) % SumGroup<Real>::pairs == 0 || j + 1 == H) {
+                        s_nout[s] += dens;
+                        dens = Real(0);
+                    }
+                } else {
+                    s_nout[s] += op.x + om.x;
+                }
+            }
         }
     }
     if (STAGE != 0 && a.periodic && owner && (i < kHalo || i >= a.nx - kHalo)) {
@@ -799,15 +893,22 @@ __device__ __forceinline__ void stage_tile(const StageArgs &a, const int64_t i0,
 
 // FP32: QL_STAGE_MINBLOCKS_F32 CTAs per SM up to Q = 32; Q = 40 holds twice the
 // Hermite coefficients and 80 KB of staged rows, and runs 2 CTAs per SM.
+// FP64: 4-warp tiles (67 KB of staged rows at Q = 32), three CTAs per SM up to
+// Q = 32 (168 registers), two at Q = 40: with one 8-warp CTA per SM (2 warps to
+// an issue slot) the FP64 pipe was 66 % busy and the integer WENO-5 chains 21 %
+// of the issue slots, each waiting for the other.
 template <typename Real, int Q>
 struct StageOccupancy {
-    static constexpr int value = sizeof(Real) == 4 ? (Q > 32 ? 2 : QL_STAGE_MINBLOCKS_F32) : 1;
+    static constexpr int value = sizeof(Real) == 4 ? (Q > 32 ? 2 : QL_STAGE_MINBLOCKS_F32) : (Q > 32 ? 2 : 3);
 };
+template <typename Real>
+QL_HD constexpr int stage_warps() { return sizeof(Real) == 8 ? kWarpsF64 : kWarps; }
 
 // One Runge-Kutta stage over a whole domain: CTA b updates tile b, or in FP64
 // with a.vsplit > 1 the velocity range b % vsplit of tile b / vsplit.
 template <typename Real, int Q, int STAGE, bool RET>
-__global__ void __launch_bounds__(kThreads, StageOccupancy<Real, Q>::value) fdlb_stage_kernel(StageArgs a)
+__global__ void __launch_bounds__(32 * stage_warps<Real>(), StageOccupancy<Real, Q>::value)
+    fdlb_stage_kernel(StageArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t mbar;
@@ -825,7 +926,8 @@ __global__ void __launch_bounds__(kThreads, StageOccupancy<Real, Q>::value) fdlb
     const int vs = sizeof(Real) == 8 ? a.vsplit : 1;
     const int64_t tile = int64_t(blockIdx.x) / vs;
     const int part = int(int64_t(blockIdx.x) - tile * vs);
-    stage_tile<Real, Q, STAGE, kWarps, RET>(a, tile * kTile, smem_raw, &mbar, 0u, part, vs);
+    constexpr int W = stage_warps<Real>();
+    stage_tile<Real, Q, STAGE, W, RET>(a, tile * TileShape<W>::tile, smem_raw, &mbar, 0u, part, vs);
 }
 
 // ---------------------------------------------------------------------------

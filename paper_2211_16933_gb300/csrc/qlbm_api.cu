@@ -17,7 +17,6 @@
 #include "../../include/qlbm_io.h"
 #include "qlbm_host.h"
 #include "qlbm_internal.h"
-#include "qlbm_lq.h"
 
 using namespace qlbm;
 
@@ -30,7 +29,12 @@ struct ql_ctx {
     std::vector<double> p, w;  // velocity set (Q)
     // velocity sets without compiled tiled kernels run on the generic FP64 path
     bool lq = false;
-    double *d_lqtab = nullptr, *d_lqmom = nullptr, *d_lqcoef = nullptr;
+    double *d_lqtab = nullptr;
+    // small FP64 domains, and every domain of those sets: stages as two launches with
+    // the per-cell quantities in memory (fdlb_cells.cuh), ccols cells at a time
+    bool cells = false;
+    void *d_coef = nullptr, *d_ch = nullptr;
+    int64_t ccols = 0;
     cudaStream_t stream = nullptr;
     ql_alloc_fn alloc = nullptr;
     ql_free_fn free_fn = nullptr;
@@ -69,6 +73,13 @@ struct ql_ctx {
     unsigned run_stages = 0;
     std::string err;
 };
+
+// FP64 domains of up to this many cells run their stages as two launches
+// (fdlb_cells.cuh) on velocity sets with tiles too; the per-cell buffers hold as
+// many cells, and other velocity sets run larger domains in chunks of them.  At
+// 131072 cells both forms take the same time (Q = 8: 438 and 447 us per step,
+// Q = 16: 785 and 794).
+constexpr int64_t kCellChunk = 131072;
 
 static std::string g_create_error;
 static std::mutex g_mutex;
@@ -147,6 +158,7 @@ static void dev_free(ql_ctx *c, void *p)
 }
 
 static FmArgs fm_args(ql_ctx *c);
+static cudaError_t fm_average(ql_ctx *c);
 
 // The buffer holding the current state psi^n, and the one the next step's
 // first and last stages write.
@@ -185,34 +197,33 @@ static StageArgs stage_args(const ql_ctx *c, const void *in, const void *base, v
 
 static cudaError_t stage(ql_ctx *c, int s, const void *in, const void *base, void *out)
 {
-    if (c->lq) {
-        LqArgs l;
-        l.in = in;
-        l.base = base;
-        l.out = out;
-        l.nx = c->nx;
-        l.stride = c->stride;
-        l.Q = c->Q;
-        l.periodic = c->periodic;
-        l.pr_mode = c->pr_mode;
-        l.enskog = c->enskog;
-        l.inv_dx = 1.0 / c->dx;
-        l.dt = c->dt;
-        l.eta0 = c->eta0;
-        l.inv_rho_ref = 1.0 / c->rho_ref;
-        l.tau_pref = c->tau_pref;
-        l.pr_const = c->pr_const;
-        l.tab = c->d_lqtab;
-        l.mom = c->d_lqmom;
-        l.coef = c->d_lqcoef;
-        l.err = c->d_err;
-        if (c->chi_mode == QL_CHI_RET_FM) {
-            // each stage averages the densities of its own input (its moments kernel writes them)
-            FmArgs f = fm_args(c);
-            f.n = c->d_lqmom + kHalo;
-            return launch_lq_stage_ret(s, l, f, c->stream);
+    if (c->cells) {
+        const bool ret = c->chi_mode == QL_CHI_RET_FM;
+        CellArgs k;
+        k.a = stage_args(c, in, base, out);
+        k.tab = c->d_lqtab;
+        k.coef = c->d_coef;
+        k.ch = c->d_ch;
+        k.K = c->d_fmk;
+        k.cs = c->ccols;
+        k.Q = c->Q;
+        k.stage = s;
+        k.W = c->fm_w;
+        k.gpairs = 0;
+        k.i0 = k.i1 = 0;
+        for (int g = 0; g < 6; ++g) k.ghost[g] = 0.0;
+        if (ret) {
+            const FmArgs f = fm_args(c);
+            for (int g = 0; g < 6; ++g) k.ghost[g] = f.ghost[g];
+            if (c->fm_w > kCellBall) {  // each stage averages the densities of its own input
+                cudaError_t e = c->lq ? launch_lq_density(c->Q, in, c->nx, c->stride, static_cast<double *>(c->d_n), c->stream)
+                                      : launch_density_f64(c->Q, in, c->nx, c->stride, c->d_n, c->stream);
+                if (e == cudaSuccess) e = fm_average(c);
+                if (e != cudaSuccess) return e;
+                k.a.nbar = c->d_nbar;
+            }
         }
-        return launch_lq_stage(s, l, c->stream);
+        return launch_cell_stage(k, ret, c->stream);
     }
     StageArgs a = stage_args(c, in, base, out);  // the launcher picks the FP64 split
     const bool ret = c->chi_mode == QL_CHI_RET_FM;
@@ -248,11 +259,11 @@ static cudaError_t fm_average(ql_ctx *c)
     return c->precision == QL_FP32 ? launch_fm_f32(f, c->stream) : launch_fm_f64(f, c->stream);
 }
 
-// chi_RET-FM: densities of the current state psi^n, then nbar (the generic
-// large-Q path forms nbar inside each stage instead).
+// chi_RET-FM: densities of the current state psi^n, then nbar (the two-launch
+// stages form nbar of their own input instead).
 static cudaError_t refresh_nbar(ql_ctx *c)
 {
-    if (c->chi_mode != QL_CHI_RET_FM || c->lq) return cudaSuccess;
+    if (c->chi_mode != QL_CHI_RET_FM || c->cells) return cudaSuccess;
     cudaError_t e = c->precision == QL_FP32 ? launch_density_f32(c->Q, state_buf(c), c->nx, c->stride, c->d_n, c->stream)
                                             : launch_density_f64(c->Q, state_buf(c), c->nx, c->stride, c->d_n, c->stream);
     return e == cudaSuccess ? fm_average(c) : e;
@@ -308,8 +319,8 @@ static void destroy_buffers(ql_ctx *c)
     dev_free(c, c->d_n);
     dev_free(c, c->d_nbar);
     dev_free(c, c->d_lqtab);
-    dev_free(c, c->d_lqmom);
-    dev_free(c, c->d_lqcoef);
+    dev_free(c, c->d_coef);
+    dev_free(c, c->d_ch);
 }
 
 extern "C" {
@@ -440,11 +451,16 @@ ql_status ql_create(const ql_velset *vs, const ql_grid *grid, double denseness, 
         e = cudaMemsetAsync(c->d_done, 0, bytes, c->stream);
         if (e != cudaSuccess) return bail(QL_ECUDA, std::string("run counters: ") + cudaGetErrorString(e));
     }
+    c->cells = c->lq || (!c->fault && c->precision == QL_FP64 && c->nx <= kCellChunk);
+    if (c->cells) {
+        c->ccols = std::min<int64_t>((c->nx + 31) / 32 * 32, kCellChunk);
+        c->d_coef = dev_alloc(c, 5 * size_t(c->ccols) * c->elem);
+        c->d_ch = dev_alloc(c, size_t(c->Q / 2) * size_t(c->ccols) * c->elem);
+        if (!c->d_coef || !c->d_ch) return bail(QL_ENOMEM, "per-cell buffer allocation failed");
+    }
     if (c->lq) {
         c->d_lqtab = static_cast<double *>(dev_alloc(c, sizeof(double) * lqtab.size()));
-        c->d_lqmom = static_cast<double *>(dev_alloc(c, sizeof(double) * 6 * ncol));
-        c->d_lqcoef = static_cast<double *>(dev_alloc(c, sizeof(double) * 9 * c->nx));
-        if (!c->d_lqtab || !c->d_lqmom || !c->d_lqcoef) return bail(QL_ENOMEM, "large-Q buffer allocation failed");
+        if (!c->d_lqtab) return bail(QL_ENOMEM, "large-Q table allocation failed");
         e = cudaMemcpyAsync(c->d_lqtab, lqtab.data(), sizeof(double) * lqtab.size(), cudaMemcpyHostToDevice, c->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);  // lqtab goes out of scope
         if (e != cudaSuccess) return bail(QL_ECUDA, std::string("large-Q tables: ") + cudaGetErrorString(e));
@@ -499,7 +515,7 @@ ql_status ql_create(const ql_velset *vs, const ql_grid *grid, double denseness, 
 // stage is averaged).  The caller flips cur afterwards when the step rotates.
 static cudaError_t enqueue_step(ql_ctx *c, int cur)
 {
-    const bool ret = c->chi_mode == QL_CHI_RET_FM && !c->lq;
+    const bool ret = c->chi_mode == QL_CHI_RET_FM && !c->cells;
     void *S = c->buf[cur], *T1 = c->buf[1 - cur], *T2 = c->buf[2];
     cudaError_t e = stage(c, 1, S, S, T1);
     if (e == cudaSuccess && ret) e = fm_average(c);

@@ -46,6 +46,8 @@ static_assert(kSeg == kThreads, "one staged cell per thread in the moment phase"
 // nx + kHalo) of row k sits at pair k * stride + kHalo + i.  stride covers
 // every staged segment of the last tile and is a multiple of 32 pairs.
 inline int64_t num_tiles(int64_t nx) { return (nx + kTile - 1) / kTile; }
+// FP64 stage kernels: 4-warp tiles, three CTAs to an SM (fdlb_kernels.cuh, StageOccupancy).
+constexpr int kWarpsF64 = 4;
 // Any tile of at most 248 cells staged from any start i0 < nx stays inside the
 // row: (i0 + tile + 2 kHalo) - (-kHalo) <= nx + 256 + kHalo.
 inline int64_t row_stride(int64_t nx) { return (nx + 256 + 2 * kHalo + 31) / 32 * 32; }
@@ -73,6 +75,12 @@ QL_HD constexpr TabView tab_view(int Q)
 {
     return TabView{tab_offset(Q), tab_offset(Q) + Q, tab_offset(Q) + 2 * Q, tab_offset(Q) + 3 * Q,
                    tab_offset(Q) + 3 * Q + Q * Q, tab_offset(Q) + 4 * Q + Q * Q};
+}
+
+// The same layout for a table of its own.
+QL_HD constexpr TabView tab_view0(int Q)
+{
+    return TabView{0, Q, 2 * Q, 3 * Q, 3 * Q + Q * Q, 4 * Q + Q * Q};
 }
 
 struct StageArgs {
@@ -216,23 +224,27 @@ struct MomentArgs {
 };
 constexpr int kMomThreads = 256;
 inline int64_t moment_blocks(int64_t nx) { return (nx + kMomThreads - 1) / kMomThreads; }
-// Generic-Q FP64 path (velocity sets without compiled kernels).  Per stage:
-// cell moments of every column, per-cell collision coefficients, then one
-// thread per (cell, velocity) for fluxes, equilibrium and update.  tab holds
-// tab_view(Q) with offset 0; mom 6 x (nx + 2 kHalo) doubles (n, u, T, q, ln n,
-// ln T); coef 9 x nx doubles.
-struct LqArgs {
-    const void *in;
-    const void *base;
-    void *out;
-    int64_t nx, stride;
-    int Q, periodic, pr_mode, enskog;
-    double inv_dx, dt, eta0, inv_rho_ref, tau_pref, pr_const;
+// One FP64 stage as two launches with the per-cell quantities in memory between
+// them (fdlb_cells.cuh): small domains, and velocity sets without compiled tiles (tab
+// != null: FP64 tables laid out as tab_view0).  a: as for the stage kernels (a.nbar
+// is read for chi_RET-FM balls of more than kCellBall cells).  coef: 5 x cs pairs,
+// ch: Q / 2 x cs pairs; the stage runs in chunks of cs cells (i0, i1 and gpairs are
+// set by the launcher).  K, ghost: the ball's 2 W + 1 weights and
+// the fixed ghost densities, as in FmArgs.
+constexpr int kCellBall = 5;
+struct CellArgs {
+    StageArgs a;
     const double *tab;
-    double *mom, *coef;
-    unsigned *err;
+    void *coef, *ch;
+    const double *K;
+    int64_t cs, i0, i1;
+    int Q, stage, W;
+    int gpairs;  // velocity pairs per moment group
+    double ghost[6];
 };
-cudaError_t launch_lq_stage(int stage, const LqArgs &a, cudaStream_t s);
+cudaError_t launch_cell_stage(CellArgs s, bool ret, cudaStream_t st);
+// Density sum_k phi_k of every interior cell for any Q (FP64), in the order of the cell kernel.
+cudaError_t launch_lq_density(int Q, const void *psi, int64_t nx, int64_t stride, double *n, cudaStream_t s);
 cudaError_t launch_lq_init(int Q, const double *rho, const double *u, const double *T, void *psi, int64_t nx,
                            int64_t stride, const double *tab, cudaStream_t s);
 cudaError_t launch_lq_moments(int Q, const MomentArgs &a, const double *tab, cudaStream_t s);

@@ -63,7 +63,7 @@ __device__ __forceinline__ void i64_indicator_(int64_t s, int64_t d, uint64_t &B
     e = unsigned(2 * sh + k);
 }
 
-// The face value f0 + (sum_q w_q (F^q - f0)) / sum_q w_q of App. A.2 from the
+// N face values h[e] = f0 + (sum_q w_q (F^q - f0)) / sum_q w_q of App. A.2 from the
 // differences a = f_{i-2} - f_{i-1}, b = f_i - f_{i-1}, g = f_{i+1} - f_i and
 // c = f_{i+2} - f_{i+1}, with w_q = delta_q prod_{r != q} beta_r^2 (rows of
 // Table weno_x with zero indicators included: weights of zero indicators
@@ -71,43 +71,84 @@ __device__ __forceinline__ void i64_indicator_(int64_t s, int64_t d, uint64_t &B
 // indicators, up to a common factor, are sums of two squares:
 //   (a + 11/8 b)^2 + 39/64 b^2,  (g - 5/8 b)^2 + 39/64 b^2,  (c - 11/8 g)^2 + 39/64 g^2,
 // and 6 (F^q - f0) = 2a + 5b, b + 2g, 4g - c.  A non-finite difference gives NaN.
-__device__ __forceinline__ double weno5_face_i64(double a, double b, double g, double c, double f0)
+// One face value is a chain of about 600 instructions with little of it independent;
+// the N are written side by side, step by step, so that a lone warp has N
+// chains in flight (N = 2 in the small-domain kernels, 7 - 10 % of a step; the tile
+// kernels, with three warps to an issue slot, run 5 % slower so and take N = 1).
+template <int N>
+__device__ __forceinline__ void weno5_faces_i64(const double (&a)[N], const double (&b)[N], const double (&g)[N],
+                                                const double (&c)[N], const double (&f0)[N], double (&h)[N])
 {
     const uint32_t kAbs = 0x7FFFFFFFu;
-    const uint32_t h = max(max(uint32_t(__double2hiint(a)) & kAbs, uint32_t(__double2hiint(b)) & kAbs),
-                           max(uint32_t(__double2hiint(g)) & kAbs, uint32_t(__double2hiint(c)) & kAbs));
-    const int E = max(int(h >> 20), 1);
-    const int64_t xa = i64_fix_(a, E), xb = i64_fix_(b, E), xg = i64_fix_(g, E), xc = i64_fix_(c, E);
-    uint64_t B1, B2, B3;
-    unsigned e1, e2, e3;
-    i64_indicator_(xa + xb + (xb >> 2) + (xb >> 3), xb, B1, e1);
-    i64_indicator_(xg - (xb >> 1) - (xb >> 3), xb, B2, e2);
-    i64_indicator_(xc - xg - (xg >> 2) - (xg >> 3), xg, B3, e3);
+    int E[N];
+    int64_t xa[N], xb[N], xg[N], xc[N];
+    uint64_t B[3][N], W[3][N], S[N];
+    unsigned e[3][N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        const uint32_t m = max(max(uint32_t(__double2hiint(a[k])) & kAbs, uint32_t(__double2hiint(b[k])) & kAbs),
+                               max(uint32_t(__double2hiint(g[k])) & kAbs, uint32_t(__double2hiint(c[k])) & kAbs));
+        E[k] = max(int(m >> 20), 1);
+    }
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        xa[k] = i64_fix_(a[k], E[k]);
+        xb[k] = i64_fix_(b[k], E[k]);
+        xg[k] = i64_fix_(g[k], E[k]);
+        xc[k] = i64_fix_(c[k], E[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < N; ++k) i64_indicator_(xa[k] + xb[k] + (xb[k] >> 2) + (xb[k] >> 3), xb[k], B[0][k], e[0][k]);
+#pragma unroll
+    for (int k = 0; k < N; ++k) i64_indicator_(xg[k] - (xb[k] >> 1) - (xb[k] >> 3), xb[k], B[1][k], e[1][k]);
+#pragma unroll
+    for (int k = 0; k < N; ++k) i64_indicator_(xc[k] - xg[k] - (xg[k] >> 2) - (xg[k] >> 3), xg[k], B[2][k], e[2][k]);
     // products of two indicators, squared, relative to the smallest indicator's
     // exponent: 1 : 6 : 3 are the ideal weights
-    const uint64_t M23 = __umul64hi(B2, B3), M13 = __umul64hi(B1, B3), M12 = __umul64hi(B1, B2);
-    const unsigned em = max(max(e1, e2), e3);
-    uint64_t W1 = __umul64hi(M23, M23) >> min(2u * (em - e1) + 5u, 63u);
-    uint64_t W2 = 6 * (__umul64hi(M13, M13) >> min(2u * (em - e2) + 5u, 63u));
-    uint64_t W3 = 3 * (__umul64hi(M12, M12) >> min(2u * (em - e3) + 5u, 63u));
-    uint64_t S = W1 + W2 + W3;  // in [2^55, 2^62.4)
-    const int k = __clz(int(S >> 32)) - 1;
-    S <<= k;
-    const int64_t N = __mul64hi(int64_t(W1 << k), 2 * xa + 5 * xb) + __mul64hi(int64_t(W2 << k), xb + 2 * xg) +
-                      __mul64hi(int64_t(W3 << k), 4 * xg - xc);
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        const unsigned em = max(max(e[0][k], e[1][k]), e[2][k]);
+        const uint64_t M23 = __umul64hi(B[1][k], B[2][k]), M13 = __umul64hi(B[0][k], B[2][k]),
+                       M12 = __umul64hi(B[0][k], B[1][k]);
+        W[0][k] = __umul64hi(M23, M23) >> min(2u * (em - e[0][k]) + 5u, 63u);
+        W[1][k] = 6 * (__umul64hi(M13, M13) >> min(2u * (em - e[1][k]) + 5u, 63u));
+        W[2][k] = 3 * (__umul64hi(M12, M12) >> min(2u * (em - e[2][k]) + 5u, 63u));
+        S[k] = W[0][k] + W[1][k] + W[2][k];  // in [2^55, 2^62.4)
+    }
+    int64_t Nm[N], d[N];
+    uint64_t x0[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        const int n = __clz(int(S[k] >> 32)) - 1;
+        S[k] <<= n;
+        Nm[k] = __mul64hi(int64_t(W[0][k] << n), 2 * xa[k] + 5 * xb[k]) +
+                __mul64hi(int64_t(W[1][k] << n), xb[k] + 2 * xg[k]) + __mul64hi(int64_t(W[2][k] << n), 4 * xg[k] - xc[k]);
+    }
     // X = 2^125 / S: x0 from the FP32 reciprocal (relative error about 2^-22),
     // then x0 (1 + d + d^2) with d = 1 - S x0 (Householder's third-order step)
-    float rf;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(float(uint32_t(S >> 32))));
-    const uint64_t x0 = uint64_t(uint32_t(rf * 2305843009213693952.0f)) << 32;
-    int64_t d = int64_t(0x2000000000000000ull - __umul64hi(S, x0));
-    const int32_t dd = int32_t(d >> 10);
-    d += (int64_t(dd) * dd) >> 41;
-    const int64_t X = int64_t(x0 + uint64_t(__mul64hi(d << 20, int64_t(x0 >> 1)) >> 16));
-    // Q = 3 (h - f0) 2^(58 - (E - 1023)): one third of the unit, by its exponent
-    const int64_t Q = __mul64hi(N << 2, X);
-    const int unit = E >= 61 ? 0x3FD55555 + ((E - 1081) << 20) : 0;
-    return fma(i64_to_double_(Q), __hiloint2double(E == 0x7FF ? 0x7FF80000 : unit, 0x55555555), f0);
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        float rf;
+        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(float(uint32_t(S[k] >> 32))));
+        x0[k] = uint64_t(uint32_t(rf * 2305843009213693952.0f)) << 32;
+        d[k] = int64_t(0x2000000000000000ull - __umul64hi(S[k], x0[k]));
+        const int32_t dd = int32_t(d[k] >> 10);
+        d[k] += (int64_t(dd) * dd) >> 41;
+    }
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        const int64_t X = int64_t(x0[k] + uint64_t(__mul64hi(d[k] << 20, int64_t(x0[k] >> 1)) >> 16));
+        // Q = 3 (h - f0) 2^(58 - (E - 1023)): one third of the unit, by its exponent
+        const int64_t Q = __mul64hi(Nm[k] << 2, X);
+        const int unit = E[k] >= 61 ? 0x3FD55555 + ((E[k] - 1081) << 20) : 0;
+        h[k] = fma(i64_to_double_(Q), __hiloint2double(E[k] == 0x7FF ? 0x7FF80000 : unit, 0x55555555), f0[k]);
+    }
+}
+__device__ __forceinline__ double weno5_face_i64(double a, double b, double g, double c, double f0)
+{
+    double h[1];
+    weno5_faces_i64<1>({a}, {b}, {g}, {c}, {f0}, h);
+    return h[0];
 }
 
 }  // namespace qlbm
