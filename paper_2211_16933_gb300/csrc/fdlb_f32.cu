@@ -8,6 +8,7 @@ static __constant__ __align__(16) float QL_TAB[kTabTotal];
 #define QL_REAL float
 #define QL_SUFFIX f32
 #include "fdlb_impl.cuh"
+#include "fdlb_narrow.cuh"
 
 namespace qlbm {
 // Per device: the kernel's shared-memory limit set, and the CTAs it holds at once.

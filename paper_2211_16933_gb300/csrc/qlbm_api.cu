@@ -58,6 +58,11 @@ struct ql_ctx {
     int chi_mode = QL_CHI_SET, fm_w = 0;
     double *d_fmk = nullptr;  // 2 fm_w + 1
     void *d_n = nullptr;      // nx values of the working precision
+    // small FP32 domains run fdlb_narrow_kernel, which reads the densities of its
+    // input while it writes those of its output: those of the state in buf[b] are
+    // in d_n (b = 0) or d_n2 (b = 1)
+    bool narrow = false;
+    void *d_n2 = nullptr;
     void *d_nbar = nullptr;   // stride values (columns -kHalo .. ; the tail past nx + kHalo unused)
     // ql_step of more than one step replays a recorded step, one recording per
     // value of cur (its launches read only buffers fixed for the context's lifetime)
@@ -80,6 +85,9 @@ struct ql_ctx {
 // 131072 cells both forms take the same time (Q = 8: 438 and 447 us per step,
 // Q = 16: 785 and 794).
 constexpr int64_t kCellChunk = 131072;
+// FP32 domains of up to this many cells run fdlb_narrow_kernel: it is ahead up to
+// 24576 cells at Q = 32 and 40 and about 16384 at Q = 8 and 16 (fdlb_narrow.cuh).
+constexpr int64_t kNarrowCells = 16384;
 
 static std::string g_create_error;
 static std::mutex g_mutex;
@@ -225,8 +233,22 @@ static cudaError_t stage(ql_ctx *c, int s, const void *in, const void *base, voi
         }
         return launch_cell_stage(k, ret, c->stream);
     }
-    StageArgs a = stage_args(c, in, base, out);  // the launcher picks the FP64 split
     const bool ret = c->chi_mode == QL_CHI_RET_FM;
+    if (c->narrow) {
+        NarrowArgs k;
+        k.a = stage_args(c, in, base, out);
+        k.f = FmArgs{};
+        if (ret) {
+            // psi^n is base: its densities, then each stage's, alternate between the two arrays
+            void *n[2] = {c->d_n, c->d_n2};
+            const int b = (base == c->buf[1]) != (s == 2);
+            k.f = fm_args(c);
+            k.f.n = n[b];
+            k.a.nout = s != 0 ? n[1 - b] : nullptr;
+        }
+        return launch_narrow_f32(c->Q, s, k, ret, c->stream);
+    }
+    StageArgs a = stage_args(c, in, base, out);  // the launcher picks the FP64 split
     a.nbar = ret ? c->d_nbar : nullptr;
     a.nout = ret && s != 0 ? c->d_n : nullptr;
     return c->precision == QL_FP32 ? launch_stage_f32(c->Q, s, a, c->stream)
@@ -264,6 +286,8 @@ static cudaError_t fm_average(ql_ctx *c)
 static cudaError_t refresh_nbar(ql_ctx *c)
 {
     if (c->chi_mode != QL_CHI_RET_FM || c->cells) return cudaSuccess;
+    if (c->narrow)  // nbar is formed inside each stage
+        return launch_density_f32(c->Q, state_buf(c), c->nx, c->stride, c->cur ? c->d_n2 : c->d_n, c->stream);
     cudaError_t e = c->precision == QL_FP32 ? launch_density_f32(c->Q, state_buf(c), c->nx, c->stride, c->d_n, c->stream)
                                             : launch_density_f64(c->Q, state_buf(c), c->nx, c->stride, c->d_n, c->stream);
     return e == cudaSuccess ? fm_average(c) : e;
@@ -317,6 +341,7 @@ static void destroy_buffers(ql_ctx *c)
     dev_free(c, c->d_done);
     dev_free(c, c->d_fmk);
     dev_free(c, c->d_n);
+    dev_free(c, c->d_n2);
     dev_free(c, c->d_nbar);
     dev_free(c, c->d_lqtab);
     dev_free(c, c->d_coef);
@@ -452,6 +477,8 @@ ql_status ql_create(const ql_velset *vs, const ql_grid *grid, double denseness, 
         if (e != cudaSuccess) return bail(QL_ECUDA, std::string("run counters: ") + cudaGetErrorString(e));
     }
     c->cells = c->lq || (!c->fault && c->precision == QL_FP64 && c->nx <= kCellChunk);
+    c->narrow = !c->lq && !c->fault && c->precision == QL_FP32 && c->nx <= kNarrowCells &&
+                (c->chi_mode == QL_CHI_SET || c->fm_w <= kNarrowBall);
     if (c->cells) {
         c->ccols = std::min<int64_t>((c->nx + 31) / 32 * 32, kCellChunk);
         c->d_coef = dev_alloc(c, 5 * size_t(c->ccols) * c->elem);
@@ -470,7 +497,8 @@ ql_status ql_create(const ql_velset *vs, const ql_grid *grid, double denseness, 
         c->d_fmk = static_cast<double *>(dev_alloc(c, sizeof(double) * (2 * c->fm_w + 1)));
         c->d_n = dev_alloc(c, real * c->nx);
         c->d_nbar = dev_alloc(c, real * c->stride);
-        if (!c->d_fmk || !c->d_n || !c->d_nbar) return bail(QL_ENOMEM, "chi_RET-FM buffer allocation failed");
+        if (c->narrow) c->d_n2 = dev_alloc(c, real * c->nx);
+        if (!c->d_fmk || !c->d_n || !c->d_nbar || (c->narrow && !c->d_n2)) return bail(QL_ENOMEM, "chi_RET-FM buffer allocation failed");
         std::vector<double> K(2 * c->fm_w + 1);
         fm_weights(c->dx, c->sigma, c->fm_w, K.data());
         e = cudaMemcpyAsync(c->d_fmk, K.data(), sizeof(double) * K.size(), cudaMemcpyHostToDevice, c->stream);
@@ -515,7 +543,7 @@ ql_status ql_create(const ql_velset *vs, const ql_grid *grid, double denseness, 
 // stage is averaged).  The caller flips cur afterwards when the step rotates.
 static cudaError_t enqueue_step(ql_ctx *c, int cur)
 {
-    const bool ret = c->chi_mode == QL_CHI_RET_FM && !c->cells;
+    const bool ret = c->chi_mode == QL_CHI_RET_FM && !c->cells && !c->narrow;
     void *S = c->buf[cur], *T1 = c->buf[1 - cur], *T2 = c->buf[2];
     cudaError_t e = stage(c, 1, S, S, T1);
     if (e == cudaSuccess && ret) e = fm_average(c);

@@ -131,6 +131,17 @@ struct FmArgs {
     double ghost[6];
 };
 
+// One FP32 stage of a small domain (fdlb_narrow.cuh).  a: as for the stage kernels
+// (a.nbar unused).  chi_RET-FM: f gives the ball of at most kNarrowBall cells
+// (f.nbar unused) and f.n the densities of the stage input; a.nout, those of its
+// output, is another buffer.
+constexpr int kNarrowBall = 16;
+struct NarrowArgs {
+    StageArgs a;
+    FmArgs f;
+};
+cudaError_t launch_narrow_f32(int Q, int stage, const NarrowArgs &s, bool ret, cudaStream_t st);
+
 // Batched form: instances packed in three arenas (psi^n, psi^(1), psi^(2)),
 // instance rows starting at pair offset `off` in each.
 struct BatchInstance {
