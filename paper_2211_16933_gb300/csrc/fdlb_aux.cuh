@@ -15,16 +15,11 @@ namespace qlbm {
 // Hermite coefficients once, then g at +p_k and -p_k from the even and odd
 // parts of the sum.
 template <typename Real, int Q>
-__global__ void fdlb_init_kernel(const double *__restrict__ rho, const double *__restrict__ u,
-                                 const double *__restrict__ T, P2<Real> *__restrict__ psi, int64_t nx,
-                                 int64_t stride, const double *__restrict__ tab)
+__device__ __forceinline__ void init_column(double uu, double TT, double n, P2<Real> *__restrict__ psi, int64_t stride,
+                                            const double *__restrict__ tab)
 {
     constexpr TabView TV = tab_view(Q);
     constexpr int H = Q / 2;
-    const int64_t ncol = nx + 2 * kHalo;
-    const int64_t c = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;  // column, cell c - kHalo
-    if (c >= ncol) return;
-    const double uu = u[c], TT = T[c], n = rho[c];
     double ch[Q];
     ch[0] = 1.0;
     ch[1] = uu;
@@ -39,9 +34,18 @@ __global__ void fdlb_init_kernel(const double *__restrict__ rho, const double *_
             o = fma(G[l + 1], ch[l + 1], o);
         }
         const double gp = n * (e + o), gm = n * (e - o);
-        psi[int64_t(H + j) * stride + c] = mk2(Real(gp), Real(2.0 * TT * gp));
-        psi[int64_t(H - 1 - j) * stride + c] = mk2(Real(gm), Real(2.0 * TT * gm));
+        psi[int64_t(H + j) * stride] = mk2(Real(gp), Real(2.0 * TT * gp));
+        psi[int64_t(H - 1 - j) * stride] = mk2(Real(gm), Real(2.0 * TT * gm));
     }
+}
+template <typename Real, int Q>
+__global__ void fdlb_init_kernel(const double *__restrict__ rho, const double *__restrict__ u,
+                                 const double *__restrict__ T, P2<Real> *__restrict__ psi, int64_t nx,
+                                 int64_t stride, const double *__restrict__ tab)
+{
+    const int64_t ncol = nx + 2 * kHalo;
+    const int64_t c = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;  // column, cell c - kHalo
+    if (c < ncol) init_column<Real, Q>(u[c], T[c], rho[c], psi + c, stride, tab);
 }
 
 template <typename Real>

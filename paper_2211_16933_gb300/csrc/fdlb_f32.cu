@@ -7,6 +7,7 @@ static __constant__ __align__(16) float QL_TAB[kTabTotal];
 }
 #define QL_REAL float
 #define QL_SUFFIX f32
+#define QL_INIT_FF  // initial states in double-FP32 (fdlb_init_ff.cuh)
 #include "fdlb_impl.cuh"
 #include "fdlb_narrow.cuh"
 

@@ -7,6 +7,9 @@
 
 #include "fdlb_kernels.cuh"
 #include "fdlb_aux.cuh"
+#ifdef QL_INIT_FF
+#include "fdlb_init_ff.cuh"
+#endif
 
 #define QL_CAT2(a, b) a##b
 #define QL_CAT(a, b) QL_CAT2(a, b)
@@ -53,6 +56,10 @@ cudaError_t QL_FN(upload_tables_)(const double *all)
     split(0.693147180559945309417232121458176568L, &lt[257].x, &lt[257].y);
     const cudaError_t e = cudaMemcpyToSymbol(QL_LOGTAB, lt, sizeof(lt));
     if (e != cudaSuccess) return e;
+#endif
+#ifdef QL_INIT_FF
+    const cudaError_t ef = upload_ff_table(all);
+    if (ef != cudaSuccess) return ef;
 #endif
     return cudaMemcpyToSymbol(QL_TAB, host, sizeof(host));
 }
@@ -227,12 +234,18 @@ cudaError_t QL_FN(launch_init_)(int Q, const double *rho, const double *u, const
     const unsigned blocks = unsigned((n + 255) / 256);
     P2<QL_REAL> *p = static_cast<P2<QL_REAL> *>(psi);
     switch (Q) {
-    case 8: fdlb_init_kernel<QL_REAL, 8><<<blocks, 256, 0, s>>>(rho, u, T, p, nx, stride, tab64); break;
-    case 16: fdlb_init_kernel<QL_REAL, 16><<<blocks, 256, 0, s>>>(rho, u, T, p, nx, stride, tab64); break;
-    case 20: fdlb_init_kernel<QL_REAL, 20><<<blocks, 256, 0, s>>>(rho, u, T, p, nx, stride, tab64); break;
-    case 24: fdlb_init_kernel<QL_REAL, 24><<<blocks, 256, 0, s>>>(rho, u, T, p, nx, stride, tab64); break;
-    case 32: fdlb_init_kernel<QL_REAL, 32><<<blocks, 256, 0, s>>>(rho, u, T, p, nx, stride, tab64); break;
-    case 40: fdlb_init_kernel<QL_REAL, 40><<<blocks, 256, 0, s>>>(rho, u, T, p, nx, stride, tab64); break;
+#ifdef QL_INIT_FF
+#define QL_INIT(Q) fdlb_init_ff_kernel<Q>
+#else
+#define QL_INIT(Q) fdlb_init_kernel<QL_REAL, Q>
+#endif
+    case 8: QL_INIT(8)<<<blocks, 256, 0, s>>>(rho, u, T, p, nx, stride, tab64); break;
+    case 16: QL_INIT(16)<<<blocks, 256, 0, s>>>(rho, u, T, p, nx, stride, tab64); break;
+    case 20: QL_INIT(20)<<<blocks, 256, 0, s>>>(rho, u, T, p, nx, stride, tab64); break;
+    case 24: QL_INIT(24)<<<blocks, 256, 0, s>>>(rho, u, T, p, nx, stride, tab64); break;
+    case 32: QL_INIT(32)<<<blocks, 256, 0, s>>>(rho, u, T, p, nx, stride, tab64); break;
+    case 40: QL_INIT(40)<<<blocks, 256, 0, s>>>(rho, u, T, p, nx, stride, tab64); break;
+#undef QL_INIT
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
