@@ -88,6 +88,24 @@ __device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t da, uint64_t
                  "l"(da), "l"(db), "r"(idesc), "r"(accumulate)
                  : "memory");
 }
+// The same issued by the thread with `leader` set while its whole warp runs the code around it: the
+// operands then stay in uniform registers, which the instruction reads (in a branch of one
+// thread each is moved there first).
+__device__ __forceinline__ void umma_bf16_leader(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc,
+                                                 int accumulate, int leader)
+{
+    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+                 "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
+                 "l"(da), "l"(db), "r"(idesc), "r"(accumulate), "r"(leader)
+                 : "memory");
+}
+// 1 in one thread of the (converged) warp.
+__device__ __forceinline__ int elect_one()
+{
+    int e;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(e));
+    return e;
+}
 __device__ __forceinline__ bool mbar_test(uint64_t *bar, uint32_t parity)
 {
     uint32_t ok;
@@ -178,6 +196,21 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t by
                      smem_u32(dst)),
                  "l"(src), "r"(bytes), "r"(smem_u32(bar))
                  : "memory");
+}
+// The same for data whose last use this is (marked first for eviction from L2).
+__device__ __forceinline__ void bulk_g2s_last(void *dst, const void *src, uint32_t bytes, uint64_t *bar)
+{
+    uint64_t pol;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
+    asm volatile(
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;" ::
+            "r"(smem_u32(dst)),
+        "l"(src), "r"(bytes), "r"(smem_u32(bar)), "l"(pol)
+        : "memory");
+}
+__device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes)
+{
+    asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
 }
 __device__ __forceinline__ void mbar_arrive_tx(uint64_t *bar, uint32_t bytes)
 {
@@ -458,52 +491,163 @@ __global__ void __launch_bounds__(role_threads(conv_epi_warps(COUT)), 2)
     }
 }
 
-// Weight and bias gradients of one layer on the tensor cores:
+// Weight and bias gradients of the layers on the tensor cores:
 //   dW[co][j][ci] = sum_{b,x} dz[b][x][co] in[b][x + j - 2][ci],  db[co] = sum dz[b][x][co].
-// Per tap j a GEMM over K = positions, accumulated in TMEM over every (sample,
-// 128-position tile) item of the CTA: the operand with 64 channels is A (M =
-// 64), the other B (N = its channel count), D_j in TMEM columns [j N, (j + 1) N).
-// Both operands are MN-major in the no-swizzle canonical layout, staged as
+// Per tap j a GEMM over K = positions, accumulated in TMEM over the (sample, 128-position
+// tile) items part, part + nparts, ... of a layer: the operand with 64 channels is A (M =
+// 64), the other B (N = its channel count), D_j in TMEM columns [j N, (j + 1) N) of the
+// job's accumulator.  Both operands are MN-major in the no-swizzle canonical layout, staged as
 // [chunk of 8 channels][position][8] (a bulk copy per chunk of the
 // chunk-major tensors): 8 consecutive positions of a chunk are one core
 // matrix, the next 8 positions follow at 128 bytes (LBO) and the next chunk at
 // a whole chunk's rows (SBO); tap j of the input window is the same descriptor
-// moved by j rows.  An M = 64 accumulator keeps row m in TMEM lane
-// 32 (m / 16) + m % 16.  The copy warp fills kWgradStages stages ahead of the
-// tensor cores; a stage is free again once its products have completed and
-// the epilogue warps have added its dz tile into their bias-gradient partial
-// sums (empty: one commit + 128 arrivals).  Each CTA writes one partial
-// [co][5 cin] + [co]; reduce_partials_kernel sums the partials in a fixed
-// order.  A wait that gives up sets bit 1 of *err and ends the CTA's work.
+// moved by j rows.  A product costs much the same for N = 16 to 128 (45 to 60 cycles
+// measured), so the window is staged more than once, one position apart: twice for 64
+// input channels (taps in pairs, N = 128: 3 products per 16 positions instead of 5), once
+// per tap for 16 (N = 80: 1 instead of 5).  An M = 64 accumulator keeps row m in TMEM lane
+// 32 (m / 16) + m % 16.
+//
+// One launch takes every layer: a CTA per SM walks jobs (layer, part) as one pipeline.  The
+// copy warps fill kWgradStages stages ahead of the tensor cores, across jobs; a stage is
+// free again once its products have completed and the bias warps have added its dz
+// tile into their sums (empty: one commit + 128 arrivals; warps of their own, so that reading an
+// accumulator out holds up no stage).  The
+// accumulator of a 64 x 64 layer takes 320 TMEM columns, the others 80: one of the former and
+// two of the latter are held, so the epilogue of a job runs beside the products of the next
+// one of the other kind (the jobs are ordered alternately).  Batch 256, 512 positions, five
+// layers: 41 us, where a launch per layer took 92 (13 to 22 each); of this, loads
+// marked for eviction (the partials then stay in L2 for their sum) and a copy warp per stage
+// gave 4, products issued by a converged warp 13.  A job writes its partial as
+// [column j N + n][m], 64 consecutive bytes per warp and column, then the 64 or 16 bias sums;
+// reduce_partials_kernel sums the partials in a fixed order.  A wait that gives up sets bit
+// 1 of *err and ends the CTA's work.
+constexpr int kChainLayers = 8;  // layers of one launch (weight gradients, whole-network kernel)
+struct WgradEntry {  // parts part0 .. part0 + njobs - 1 (of nparts) of a layer
+    const bf16 *dz, *in;
+    float *partial;  // [nparts][wgrad_len]
+    int cin, cout;   // padded
+    int part0, nparts, njobs;
+};
+struct WgradArgs {
+    WgradEntry E[2 * kChainLayers];
+    int ne, njobs;
+    const int *periodic;
+    int X, ntiles;
+    unsigned *err;
+};
+__host__ __device__ constexpr int wgrad_cols(int cin, int cout) { return kTaps * (cout == 64 ? cin : cout); }
+__host__ __device__ constexpr int wgrad_len(int cin, int cout) { return wgrad_cols(cin, cout) * 64 + cout; }
+constexpr int kWgradInWarps = kWgradStages;  // copy warps of the input windows
+constexpr int kWgradThreads = 32 * (2 * kWgradEpiWarps + kWgradInWarps + 2);
+constexpr int kWgradStageBytes = 16 * (8 * kConvM + 16 * (kConvM + kTaps - 1));  // dz and two windows of 64 channels
+// Accumulators: 0 of a 64 x 64 layer, 1 and 2 of the others.
+__device__ __forceinline__ uint32_t wgrad_acc_col(int acc) { return acc == 0 ? 0u : (acc == 1 ? 320u : 400u); }
+
+// The jobs of a CTA in order: entry, part, accumulator and how often that was used before.
+struct WgradWalk {
+    int job, e = 0, job0 = 0, big = 0, small = 0, acc = 0, use = 0, part = 0;
+    __device__ __forceinline__ explicit WgradWalk() : job(int(blockIdx.x)) {}
+    __device__ __forceinline__ bool valid(const WgradArgs &a)
+    {
+        if (job >= a.njobs) return false;
+        while (job >= job0 + a.E[e].njobs) job0 += a.E[e++].njobs;
+        part = a.E[e].part0 + job - job0;
+        if (a.E[e].cin == 64 && a.E[e].cout == 64) {
+            acc = 0;
+            use = big++;
+        } else {
+            acc = 1 + (small & 1);
+            use = small++ >> 1;
+        }
+        job += int(gridDim.x);
+        return true;
+    }
+};
+
+// The products of one item (dz tile and input window staged at ad).
 template <int CIN, int COUT>
-__global__ void __launch_bounds__(role_threads(kWgradEpiWarps), 1)
-    wgrad_kernel(const bf16 *__restrict__ dz, const bf16 *__restrict__ in, const int *__restrict__ periodic, int X,
-                 int ntiles, float *__restrict__ partial, unsigned *__restrict__ err)
+__device__ __forceinline__ void wgrad_products(uint32_t tacc, uint32_t ad, bool first, int leader)
 {
     static_assert((COUT == 64 && (CIN == 16 || CIN == 64)) || (COUT == 16 && CIN == 64), "layer shapes");
-    constexpr bool DZ_A = COUT == 64;           // A = dz (M = cout); else A = input window (M = cin)
-    constexpr int NB = DZ_A ? CIN : COUT;       // N of one tap
-    constexpr int KCD = COUT / 8, KCI = CIN / 8;
-    constexpr int RD = kConvM, RI = kConvM + kTaps - 1;  // staged positions of dz and of the input window
-    constexpr uint32_t SD = RD * 16, SI = RI * 16;       // chunk strides (bytes)
-    constexpr int NTOT = kTaps * NB, NS = kWgradStages;
-    constexpr int kCopy = kWgradEpiWarps, kMma = kWgradEpiWarps + 1;
-    constexpr uint32_t NCOL = NTOT <= 32 ? 32 : (NTOT <= 64 ? 64 : (NTOT <= 128 ? 128 : (NTOT <= 256 ? 256 : 512)));
-    constexpr int kStage = KCD * RD * 8 + KCI * RI * 8;  // bf16 per stage
-    // bias gradient: epilogue warp w sums dz chunks w and w + 4 (those below KCD),
-    // lane l the rows l, l + 32, l + 64, l + 96 of each tile
-    constexpr int DBC = KCD > 4 ? 2 : 1;
+    constexpr uint32_t SD = kConvM * 16, SI = (kConvM + kTaps - 1) * 16;  // chunk strides (bytes)
+    // descriptors move by their address field (16-byte units: k0 + j rows, no carry out of it)
+    const uint64_t d0 = umma_desc(ad, 128, SD), i0 = umma_desc(ad + (COUT / 8) * SD, 128, CIN == 16 ? SD : SI);
+    // MN-major A and B, M = 64
+    constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | (uint32_t(64 >> 4) << 24);
+    auto mma = [&](uint32_t col, uint64_t da, uint64_t db, int N, int k0) {
+        umma_bf16_leader(tacc + col, da, db, idesc | (uint32_t(N >> 3) << 17), !first || k0 > 0, leader);
+    };
+#pragma unroll
+    for (int k0 = 0; k0 < kConvM; k0 += 16) {
+        const uint64_t dd = d0 + k0;
+        if constexpr (COUT == 16) {  // A = input window (M = cin)
+#pragma unroll
+            for (int j = 0; j < kTaps; ++j) mma(j * 16, i0 + (k0 + j), dd, 16, k0);
+        } else if constexpr (CIN == 16) {  // five windows, one per tap: N = 80
+            mma(0, dd, i0 + k0, kTaps * 16, k0);
+        } else {  // two windows, one position apart: taps in pairs, N = 128
+            mma(0, dd, i0 + k0, 128, k0);
+            mma(128, dd, i0 + (k0 + 2), 128, k0);
+            mma(256, dd, i0 + (k0 + 4), 64, k0);
+        }
+    }
+}
+
+// Rows x0 - halo .. (rows of them) of sample b into a stage, as fill_rows but without arriving on *full: the
+// bulk copies first (lane 0, their bytes added to the phase), then the rows outside the sample.
+template <int C>
+__device__ __forceinline__ void wgrad_rows(bf16 *dst, const bf16 *src, int b, int x0, int halo, int rows, int X,
+                                           int mode, int lane, uint64_t *full)
+{
+    constexpr int KC = C / 8;
+    const int first = x0 - halo;
+    // inside [lo, hi), empty where the rows begin beyond the sample
+    const int lo = first < 0 ? 0 : first, hi = max(lo, first + rows > X ? X : first + rows);
+    const int nl = lo - first, nr = first + rows - hi;
+    if (hi > lo) {
+        const uint32_t bytes = uint32_t(hi - lo) * 16u;
+        if (lane == 0) mbar_expect_tx(full, KC * bytes);
+        __syncwarp();
+        if (lane < KC)
+            bulk_g2s_last(dst + (lane * rows + nl) * 8, src + cm_index(b, lo, lane * 8, C, X, 8), bytes, full);
+    }
+    for (int e = lane; e < (nl + nr) * KC; e += 32) {
+        const int r = e / KC, c = e % KC, p = r < nl ? r : (hi - first) + (r - nl);
+        bool inside;
+        const int x = wrap_pos(first + p, X, mode, &inside);
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (inside) v = *reinterpret_cast<const uint4 *>(src + cm_index(b, x, c * 8, C, X, 8));
+        *reinterpret_cast<uint4 *>(dst + (c * rows + p) * 8) = v;
+    }
+}
+__device__ __forceinline__ void wgrad_filled(uint64_t *full)
+{
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // plain stores before the tensor cores' reads
+    __syncwarp();
+    mbar_arrive(full);
+}
+
+__global__ void __launch_bounds__(kWgradThreads, 1) wgrad_kernel(const __grid_constant__ WgradArgs a)
+{
+    constexpr int NS = kWgradStages, NACC = 3, RD = kConvM;
+    // warps: TMEM lane quarters 0 - 3, bias sums, copies (dz; input windows of every fourth item: the
+    // rows beyond a sample's ends come through registers, a round trip to memory each), products
+    constexpr int kBias = kWgradEpiWarps, kCopy = 2 * kWgradEpiWarps, kMma = kCopy + 1 + kWgradInWarps;
     extern __shared__ __align__(128) unsigned char smem[];
-    bf16 *const stage_base = reinterpret_cast<bf16 *>(smem);
-    __shared__ __align__(8) uint64_t full[NS], empty[NS], done;
+    __shared__ __align__(8) uint64_t full[NS], empty[NS], tfull[NACC], tempty[NACC], done;
     __shared__ uint32_t s_taddr;
     __shared__ int s_abort;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const int tiles = (X + kConvM - 1) / kConvM;
+    const int tiles = (a.X + kConvM - 1) / kConvM;
+    auto stage = [&](int s) { return reinterpret_cast<bf16 *>(smem + s * kWgradStageBytes); };
     if (t == 0) {
         for (int s = 0; s < NS; ++s) {
             mbar_init(&full[s], 64);
             mbar_init(&empty[s], 1 + 32 * kWgradEpiWarps);
+        }
+        for (int k = 0; k < NACC; ++k) {
+            mbar_init(&tfull[k], 1);
+            mbar_init(&tempty[k], 32 * kWgradEpiWarps);
         }
         mbar_init(&done, 1);
         s_abort = 0;
@@ -511,7 +655,7 @@ __global__ void __launch_bounds__(role_threads(kWgradEpiWarps), 1)
     }
     if (warp == kMma) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_taddr)),
-                     "r"(NCOL)
+                     "r"(512)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -522,153 +666,164 @@ __global__ void __launch_bounds__(role_threads(kWgradEpiWarps), 1)
     if (t == 0) pdl_trigger();
     const uint32_t taddr = s_taddr;
     volatile int *const abort = &s_abort;
-    int nit = 0;  // items of this CTA
-    for (int item = blockIdx.x; item < ntiles; item += gridDim.x) ++nit;
-    if (warp == kCopy) {
-        // dz rows x0 .. x0 + 127 (zero beyond the sample), input window rows x0 - 2 ..
-        // x0 + 129 (periodic or replicated ends): two fills, 64 arrivals on full
-        int it = 0;
-        for (int item = blockIdx.x; item < ntiles; item += gridDim.x, ++it) {
-            const int s = it % NS;
-            if (it >= NS && !mbar_wait(&empty[s], (it / NS - 1) & 1, abort)) {
-                give_up(abort, err);
-                break;
+    int it = 0;  // items of this CTA so far, over all its jobs: stage it % NS
+    WgradWalk w;
+    if (warp >= kCopy && warp < kMma) {
+        const int mine = warp - kCopy;  // 0: dz; else input windows of items it = mine - 1 (mod kWgradInWarps)
+        bool ok = true;
+        while (ok && w.valid(a)) {
+            const WgradEntry &E = a.E[w.e];
+            for (int item = w.part; item < a.ntiles; item += E.nparts, ++it) {
+                if (mine && it % kWgradInWarps != mine - 1) continue;
+                const int s = it % NS, b = item / tiles, x0 = (item % tiles) * kConvM;
+                const int mode = mine && a.periodic[b] != 0 ? PAD_PERIODIC : PAD_REPLICATE;
+                if (it >= NS && !mbar_wait(&empty[s], (it / NS - 1) & 1, abort)) {
+                    give_up(abort, a.err);
+                    ok = false;
+                    break;
+                }
+                constexpr int RI = kConvM + kTaps - 1;
+                bf16 *const win = stage(s) + (E.cout / 8) * RD * 8;
+                if (mine == 0) {
+                    // dz rows x0 .. x0 + 127, zero beyond the sample
+                    if (E.cout == 16) wgrad_rows<16>(stage(s), E.dz, b, x0, 0, RD, a.X, PAD_ZERO, lane, &full[s]);
+                    else wgrad_rows<64>(stage(s), E.dz, b, x0, 0, RD, a.X, PAD_ZERO, lane, &full[s]);
+                } else if (E.cin == 16) {
+                    for (int j = 0; j < kTaps; ++j)
+                        wgrad_rows<16>(win + j * 2 * RD * 8, E.in, b, x0, 2 - j, RD, a.X, mode, lane, &full[s]);
+                } else {
+                    wgrad_rows<64>(win, E.in, b, x0, 2, RI, a.X, mode, lane, &full[s]);
+                    if (E.cout == 64) wgrad_rows<64>(win + 8 * RI * 8, E.in, b, x0, 1, RI, a.X, mode, lane, &full[s]);
+                }
+                wgrad_filled(&full[s]);
             }
-            const int b = item / tiles, x0 = (item % tiles) * kConvM;
-            bf16 *sdz = stage_base + s * kStage;
-            fill_rows<COUT>(sdz, dz, b, x0, 0, RD, X, PAD_ZERO, lane, &full[s]);
-            fill_rows<CIN>(sdz + KCD * RD * 8, in, b, x0, 2, RI, X, periodic[b] != 0 ? PAD_PERIODIC : PAD_REPLICATE,
-                           lane, &full[s]);
         }
         drain_fills(full, NS, it);
     } else if (warp == kMma) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
-                                       (uint32_t(NB >> 3) << 17) | (uint32_t(64 >> 4) << 24);  // MN-major A and B, M = 64
-            for (int it = 0; it < nit; ++it) {
-                const int s = it % NS;
-                if (!mbar_wait(&full[s], (it / NS) & 1, abort)) {
-                    give_up(abort, err);
+        {
+            const int leader = elect_one();
+            bool ok = true;
+            while (ok && w.valid(a)) {
+                const WgradEntry &E = a.E[w.e];
+                // the accumulator's previous job has been read
+                if (w.use > 0 && !__all_sync(0xffffffffu, mbar_wait(&tempty[w.acc], (w.use - 1) & 1, abort))) {
+                    give_up(abort, a.err);
                     break;
                 }
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t ad = smem_u32(stage_base + s * kStage), ai = ad + KCD * RD * 16;
-#pragma unroll
-                for (int j = 0; j < kTaps; ++j)
-#pragma unroll
-                    for (int k0 = 0; k0 < kConvM; k0 += 16) {
-                        const uint64_t dd = umma_desc(ad + k0 * 16, 128, SD);
-                        const uint64_t di = umma_desc(ai + (k0 + j) * 16, 128, SI);
-                        umma_bf16(taddr + j * NB, DZ_A ? dd : di, DZ_A ? di : dd, idesc, it > 0 || k0 > 0);
+                const uint32_t tacc = taddr + wgrad_acc_col(w.acc);
+                for (int item = w.part; item < a.ntiles; item += E.nparts, ++it) {
+                    const int s = it % NS;
+                    if (!__all_sync(0xffffffffu, mbar_wait(&full[s], (it / NS) & 1, abort))) {
+                        give_up(abort, a.err);
+                        ok = false;
+                        break;
                     }
-                umma_commit(&empty[s]);
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const uint32_t ad = smem_u32(stage(s));
+                    if (E.cout == 16) wgrad_products<64, 16>(tacc, ad, item == w.part, leader);
+                    else if (E.cin == 16) wgrad_products<16, 64>(tacc, ad, item == w.part, leader);
+                    else wgrad_products<64, 64>(tacc, ad, item == w.part, leader);
+                    if (leader) umma_commit(&empty[s]);
+                    __syncwarp();
+                }
+                if (leader) umma_commit(&tfull[w.acc]);
+                __syncwarp();
             }
-            umma_commit(&done);
-            if (!mbar_wait(&done, 0, nullptr)) give_up(abort, err);
+            // every product has landed before the accumulators are freed
+            if (leader) umma_commit(&done);
+            __syncwarp();
+            if (!mbar_wait(&done, 0, nullptr)) give_up(abort, a.err);
         }
         __syncwarp();
-    } else {
-        float db[DBC][8];
-#pragma unroll
-        for (int d = 0; d < DBC; ++d)
-#pragma unroll
-            for (int k = 0; k < 8; ++k) db[d][k] = 0.f;
+    } else if (warp >= kBias) {
+        // bias gradient: bias warp v sums dz chunks v and v + 4 (those the layer has), lane l
+        // the rows l, l + 32, l + 64, l + 96 of each tile
+        const int v = warp - kBias;
         bool ok = true;
-        for (int it = 0; it < nit; ++it) {
-            const int s = it % NS;
-            if (!mbar_wait(&full[s], (it / NS) & 1, abort)) {
-                give_up(abort, err);
-                ok = false;
-                break;
-            }
-            const bf16 *sdz = stage_base + s * kStage;
+        while (ok && w.valid(a)) {
+            const WgradEntry &E = a.E[w.e];
+            const int kcd = E.cout / 8;
+            float db[2][8];
 #pragma unroll
-            for (int d = 0; d < DBC; ++d) {
-                const int c = warp + 4 * d;
-                if (c < KCD)
+            for (int d = 0; d < 2; ++d)
 #pragma unroll
-                    for (int r = 0; r < RD; r += 32) {
-                        const uint4 u = *reinterpret_cast<const uint4 *>(sdz + (c * RD + r + lane) * 8);
-                        const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&u);
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            db[d][2 * k] += __bfloat162float(h[k].x);
-                            db[d][2 * k + 1] += __bfloat162float(h[k].y);
-                        }
-                    }
-            }
-            mbar_arrive(&empty[s]);
-        }
-        // every epilogue warp has read its last dz tile before the stage buffers
-        // are reused below (also one that gave up)
-        asm volatile("bar.sync 1, %0;" ::"n"(32 * kWgradEpiWarps) : "memory");
-        // the lane sums of each column, in a fixed order
-#pragma unroll
-        for (int d = 0; d < DBC; ++d)
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) db[d][k] += __shfl_xor_sync(0xffffffffu, db[d][k], o);
-        // the accumulators once every product of the CTA has landed
-        if (!__all_sync(0xffffffffu, ok && mbar_wait(&done, 0, abort))) {  // warp-uniform, as tcgen05.ld
-            if (ok) give_up(abort, err);
-            ok = false;
-        }
-        if (ok) {
-            // the accumulators go through shared memory (the idle stage buffers) as
-            // [co][5 cin] rows padded by one word, then out in coalesced rows
-            constexpr int RW = kTaps * CIN, RP = RW + 1;
-            static_assert(COUT * RP * 4 <= NS * kStage * 2, "transpose buffer");
-            float *T = reinterpret_cast<float *>(smem);
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // after the tensor cores' reads
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            // lane l < 16 of warp w holds row m = 16 w + l of every D_j; 64 columns per wait
-            const int m = 16 * warp + lane;
-            static_assert(NTOT % 16 == 0, "whole 16-column loads");
-#pragma unroll 1
-            for (int c0 = 0; c0 < NTOT; c0 += 64) {
-                uint32_t r[64];
-#pragma unroll
-                for (int h = 0; h < 4; ++h)
-                    if (c0 + 16 * h < NTOT) tmem_ld16(r + 16 * h, taddr + (uint32_t(warp * 32) << 16) + c0 + 16 * h);
-                tmem_wait(r);
-                if (lane < 16) {
-#pragma unroll
-                    for (int q = 0; q < 64; ++q) {
-                        const int col = c0 + q, j = col / NB, n = col % NB;  // tap j, channel n of B
-                        // DZ_A: m = co, n = ci; else m = ci, n = co
-                        const int co = DZ_A ? m : n, ci = DZ_A ? n : m;
-                        if (col < NTOT) T[co * RP + j * CIN + ci] = nit > 0 ? __uint_as_float(r[q]) : 0.f;
-                    }
+                for (int k = 0; k < 8; ++k) db[d][k] = 0.f;
+            for (int item = w.part; item < a.ntiles; item += E.nparts, ++it) {
+                const int s = it % NS;
+                if (!mbar_wait(&full[s], (it / NS) & 1, abort)) {
+                    give_up(abort, a.err);
+                    ok = false;
+                    break;
                 }
+                const bf16 *sdz = stage(s);
+#pragma unroll
+                for (int d = 0; d < 2; ++d) {
+                    const int c = v + 4 * d;
+                    if (c < kcd)
+#pragma unroll
+                        for (int r = 0; r < RD; r += 32) {
+                            const uint4 u = *reinterpret_cast<const uint4 *>(sdz + (c * RD + r + lane) * 8);
+                            const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&u);
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) {
+                                db[d][2 * k] += __bfloat162float(h[k].x);
+                                db[d][2 * k + 1] += __bfloat162float(h[k].y);
+                            }
+                        }
+                }
+                mbar_arrive(&empty[s]);
             }
-        }
-        // every epilogue warp, also one that gave up (the transpose buffer is shared)
-        asm volatile("bar.sync 1, %0;" ::"n"(32 * kWgradEpiWarps) : "memory");
-        if (ok) {
-            constexpr int RW = kTaps * CIN, RP = RW + 1;
-            const float *T = reinterpret_cast<const float *>(smem);
-            float *P = partial + size_t(blockIdx.x) * (COUT * RW + COUT);
-            static_assert(RW % 4 == 0, "rows of whole float4");
-            for (int e = 4 * t; e < COUT * RW; e += 4 * 32 * kWgradEpiWarps) {
-                const float *src = T + (e / RW) * RP + e % RW;  // four values of one row
-                *reinterpret_cast<float4 *>(P + e) = make_float4(src[0], src[1], src[2], src[3]);
-            }
+            __syncwarp();
+            // the lane sums of each column, in a fixed order
+#pragma unroll
+            for (int d = 0; d < 2; ++d)
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) db[d][k] += __shfl_xor_sync(0xffffffffu, db[d][k], o);
+            float *P = E.partial + size_t(w.part) * wgrad_len(E.cin, E.cout) + wgrad_cols(E.cin, E.cout) * 64;
             if (lane == 0)
 #pragma unroll
-                for (int d = 0; d < DBC; ++d) {
-                    const int c = warp + 4 * d;
-                    if (c < KCD)
+                for (int d = 0; d < 2; ++d) {
+                    const int c = v + 4 * d;
+                    if (c < kcd)
 #pragma unroll
-                        for (int k = 0; k < 8; ++k) P[size_t(COUT) * RW + 8 * c + k] = db[d][k];
+                        for (int k = 0; k < 8; ++k) P[8 * c + k] = db[d][k];
                 }
+        }
+    } else {
+        while (w.valid(a)) {
+            const WgradEntry &E = a.E[w.e];
+            // the accumulator once every product of the job has landed (warp-uniform, as tcgen05.ld)
+            if (!__all_sync(0xffffffffu, mbar_wait(&tfull[w.acc], w.use & 1, abort))) {
+                give_up(abort, a.err);
+                break;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const int ncol = wgrad_cols(E.cin, E.cout);
+            const uint32_t tacc = taddr + wgrad_acc_col(w.acc) + (uint32_t(warp * 32) << 16);
+            // lane l < 16 of warp w holds row m = 16 w + l
+            float *row = E.partial + size_t(w.part) * wgrad_len(E.cin, E.cout) + 16 * warp + lane;
+#pragma unroll 1
+            for (int c = 0; c < ncol; c += 80) {
+                uint32_t r[80];
+#pragma unroll
+                for (int h = 0; h < 5; ++h) tmem_ld16(r + 16 * h, tacc + c + 16 * h);
+                tmem_wait(r);
+                if (lane < 16)
+#pragma unroll
+                    for (int q = 0; q < 80; ++q) row[(c + q) * 64] = __uint_as_float(r[q]);
+                __syncwarp();
+            }
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            mbar_arrive(&tempty[w.acc]);
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == kMma) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(NCOL) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(512) : "memory");
     }
 }
 
@@ -726,40 +881,131 @@ __global__ void __launch_bounds__(256) edge_grad_kernel(const bf16 *__restrict__
     }
 }
 
-// out[i] = sum_c partial[c][i] in a fixed order.  A block of 16 warps takes 128
-// consecutive i (four per lane, 16-byte loads); warp w sums the parts c = w,
-// w + 16, ... in four interleaved running sums (independent loads in flight),
-// and the warp sums are added in warp order, so the result does not depend on
-// scheduling.  len is a multiple of 4.
+// Adam on FP32 master parameters; refreshes the bf16 weight copies and the
+// tap-flipped transposed copies used by the backward pass.
+constexpr int kAdamLayers = 8;  // layers whose bf16 copies the Adam pass refreshes itself
+struct AdamArgs {
+    float *param, *m, *v;
+    const float *grad;
+    int64_t n;
+    float lr, b1, b2, eps, c1, c2;  // c1 = 1/(1-b1^t), c2 = 1/(1-b2^t)
+    // training runs: lr, c1, c2 of step *step from device arrays (null: the scalars above)
+    const int *step;
+    const float *lr_arr, *c1_arr, *c2_arr;
+    // bf16 copies written in the same pass (nl = 0: none): layer l's W[co][j][ci]
+    // at woff[l] (cout[l] x 5 x cin[l]) into w16 and, tap-flipped and
+    // transposed, into wt16 at the same offset (both in staging order)
+    bf16 *w16, *wt16;
+    int nl;
+    int64_t woff[kAdamLayers];
+    int cout[kAdamLayers], cin[kAdamLayers];
+};
+struct AdamRates {
+    float lr, c1, c2;
+};
+__device__ __forceinline__ AdamRates adam_rates(const AdamArgs &a)
+{
+    if (!a.step) return {a.lr, a.c1, a.c2};
+    const int t = *a.step;
+    return {a.lr_arr[t], a.c1_arr[t], a.c2_arr[t]};
+}
+// The update of parameter i with gradient g; returns the new parameter.
+__device__ __forceinline__ float adam_update(const AdamArgs &a, AdamRates r, int64_t i, float g)
+{
+    const float m = a.b1 * a.m[i] + (1.f - a.b1) * g;
+    const float v = a.b2 * a.v[i] + (1.f - a.b2) * g * g;
+    a.m[i] = m;
+    a.v[i] = v;
+    const float p = a.param[i] - r.lr * (m * r.c1) / (sqrtf(v * r.c2) + a.eps);
+    a.param[i] = p;
+    return p;
+}
+// The bf16 copies of weight e of a layer at woff (cout x 5 x cin).
+__device__ __forceinline__ void store_weight(bf16 *w16, bf16 *wt16, int64_t woff, int cout, int cin, int e, float p)
+{
+    const int co = e / (kTaps * cin), j = (e / cin) % kTaps, ci = e % cin;
+    const bf16 b = __float2bfloat16(p);
+    w16[woff + wstage_index(co, j, ci, cout, cin)] = b;
+    wt16[woff + wstage_index(ci, kTaps - 1 - j, co, cin, cout)] = b;
+}
+__global__ void adam_kernel(AdamArgs a)
+{
+    pdl_wait();
+    pdl_trigger();
+    const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (i >= a.n) return;
+    const float p = adam_update(a, adam_rates(a), i, a.grad[i]);
+    for (int l = 0; l < a.nl; ++l) {
+        const int64_t e = i - a.woff[l];
+        if (e >= 0 && e < int64_t(a.cout[l]) * kTaps * a.cin[l]) {
+            store_weight(a.w16, a.wt16, a.woff[l], a.cout[l], a.cin[l], int(e), p);
+            break;
+        }
+    }
+}
+
+// Parameter i of each layer (blockIdx.y): its gradient as the sum of the layer's weight-gradient
+// partials in a fixed order, and the Adam update with it (ADAM).  A block of 16 warps
+// takes 128 values, 16 rows m of 8 consecutive columns of the partials' [column][m] layout (64
+// consecutive bytes per column read, 8 consecutive parameters written), or the bias
+// sums; warp w sums the parts c = w, w + 16, ... in four interleaved running sums
+// (independent 16-byte loads in flight), and the warp sums are added in warp order, so the
+// result does not depend on scheduling.
 constexpr int kReduceWarps = 16;
+struct ReduceArgs {
+    struct {
+        const float *partial;
+        int nparts, cout, cin;
+        int64_t goff;
+    } L[kChainLayers];
+    float *grad;
+};
+__host__ __device__ constexpr int reduce_blocks(int cin, int cout) { return wgrad_cols(cin, cout) / 2 + 1; }
 __device__ __forceinline__ float4 add4(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
-__global__ void __launch_bounds__(32 * kReduceWarps) reduce_partials_kernel(const float *__restrict__ partial,
-                                                                           int nparts, int len,
-                                                                           float *__restrict__ out)
+template <bool ADAM>
+__global__ void __launch_bounds__(32 * kReduceWarps) reduce_partials_kernel(const __grid_constant__ ReduceArgs a,
+                                                                           const __grid_constant__ AdamArgs ad)
 {
     pdl_wait();
     pdl_trigger();
     __shared__ float4 s_w[kReduceWarps][32];
+    const auto &L = a.L[blockIdx.y];
+    const int nblk = reduce_blocks(L.cin, L.cout), ncol = wgrad_cols(L.cin, L.cout);
+    if (int(blockIdx.x) >= nblk) return;
+    const bool bias = int(blockIdx.x) == nblk - 1;
+    const int col0 = int(blockIdx.x >> 2) * 8, m0 = int(blockIdx.x & 3) * 16;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int i4 = blockIdx.x * 32 + lane;  // float4 index
-    const bool ok = 4 * i4 < len;
+    const bool ok = !bias || 4 * lane < L.cout;
     const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
     float4 s[4] = {z, z, z, z};
     if (ok) {
-        const float4 *p = reinterpret_cast<const float4 *>(partial) + i4;
-        const size_t row = size_t(len) / 4;
+        const float4 *p = reinterpret_cast<const float4 *>(
+            L.partial + (bias ? ncol * 64 + 4 * lane : (col0 + (lane >> 2)) * 64 + m0 + 4 * (lane & 3)));
+        const size_t row = size_t(wgrad_len(L.cin, L.cout)) / 4;
         int c = warp;
-        for (; c + 3 * kReduceWarps < nparts; c += 4 * kReduceWarps)
+        for (; c + 3 * kReduceWarps < L.nparts; c += 4 * kReduceWarps)
 #pragma unroll
             for (int r = 0; r < 4; ++r) s[r] = add4(s[r], p[size_t(c + r * kReduceWarps) * row]);
-        for (int r = 0; c < nparts; c += kReduceWarps, ++r) s[r] = add4(s[r], p[size_t(c) * row]);
+        for (int r = 0; c < L.nparts; c += kReduceWarps, ++r) s[r] = add4(s[r], p[size_t(c) * row]);
     }
     s_w[warp][lane] = add4(add4(s[0], s[1]), add4(s[2], s[3]));
     __syncthreads();
-    if (warp == 0 && ok) {
-        float4 r = s_w[0][lane];
-        for (int k = 1; k < kReduceWarps; ++k) r = add4(r, s_w[k][lane]);
-        reinterpret_cast<float4 *>(out)[i4] = r;
+    // thread t < 128 finishes one value: column col0 + t % 8, row m0 + t / 8 (t: bias channel)
+    const int t = threadIdx.x;
+    if (t >= 128 || (bias && t >= L.cout)) return;
+    const int at = bias ? t : (t & 7) * 16 + (t >> 3);
+    float g = reinterpret_cast<const float *>(s_w[0])[at];
+    for (int k = 1; k < kReduceWarps; ++k) g += reinterpret_cast<const float *>(s_w[k])[at];
+    // column j N + n and row m: (co, ci) = (m, n) when dz was operand A, else (n, m)
+    int i = L.cout * kTaps * L.cin + t;
+    if (!bias) {
+        const int nb = ncol / kTaps, col = col0 + (t & 7), j = col / nb, n = col - j * nb, m = m0 + (t >> 3);
+        i = L.cout == 64 ? (m * kTaps + j) * L.cin + n : (n * kTaps + j) * L.cin + m;
+    }
+    a.grad[L.goff + i] = g;
+    if constexpr (ADAM) {
+        const float p = adam_update(ad, adam_rates(ad), L.goff + i, g);
+        if (ad.nl && !bias) store_weight(ad.w16, ad.wt16, L.goff, L.cout, L.cin, i, p);
     }
 }
 
@@ -835,9 +1081,9 @@ inline unsigned mse_blocks(int64_t npos) { return unsigned((npos + 255) / 256); 
 // chunk-major, padded channels zero) and per-block partial sums of the squared
 // error (256 threads, one per position).
 // y rows of the batch: y[b] directly, or y[idx[b]] of the whole data set
-// (idx already checked by pack_gather_kernel; X positions per sample).
+// (sample 0 in place of an index outside [0, n), as pack_gather_kernel; X positions per sample).
 __global__ void __launch_bounds__(256) mse_kernel(const float *__restrict__ pred, const float *__restrict__ y,
-                                                  const int32_t *__restrict__ idx, const int *__restrict__ step, int X,
+                                                  const int32_t *__restrict__ idx, const int *__restrict__ step, int64_t n, int X,
                                                   int64_t npos, int cout, const float *__restrict__ inv_out_scale,
                                                   float grad_scale, bf16 *__restrict__ dpred,
                                                   float *__restrict__ partial)
@@ -852,7 +1098,9 @@ __global__ void __launch_bounds__(256) mse_kernel(const float *__restrict__ pred
     if (pos < npos) {
         const int64_t b = pos / X;
         const int p = int(pos % X);
-        const int64_t row = (idx ? int64_t(idx[b]) : b) * X + p;
+        int64_t k = idx ? int64_t(idx[b]) : b;
+        if (idx && (k < 0 || k >= n)) k = 0;
+        const int64_t row = k * X + p;
         float g[kOutPad];
 #pragma unroll
         for (int q = 0; q < kOutPad / 4; ++q) {
@@ -904,15 +1152,15 @@ __global__ void unpack_output_kernel(const float *__restrict__ pred, int64_t npo
     y[e] = pred[cm_index(pos / X, pos % X, c, coutp, X, 4)] * out_scale[c];
 }
 
-// Mean loss of one batch from the per-block partial sums of mse_kernel, summed
-// in a fixed order by one block of 256 threads: each thread adds its strided
-// share in FP32, the thread sums are combined in FP64.
-__global__ void loss_sum_kernel(const float *__restrict__ partial, int nparts, float scale, float *__restrict__ out,
-                                const int *__restrict__ step)
+// Last launch of a training run's step: the batch's mean loss into losses[*step]
+// (losses may be null) and the step counter's advance.  The partial sums of the
+// squared error are added in a fixed order by one block of 256 threads: each
+// thread adds its strided share in FP32, the thread sums are combined in FP64.
+__global__ void loss_step_kernel(const float *__restrict__ partial, int nparts, float scale,
+                                 float *__restrict__ losses, int *__restrict__ step)
 {
     pdl_wait();
     pdl_trigger();
-    if (step) out += *step;
     __shared__ double red[256];
     // four independent running sums per thread (loads in flight), combined in order
     float s4[4] = {0.f, 0.f, 0.f, 0.f};
@@ -927,66 +1175,413 @@ __global__ void loss_sum_kernel(const float *__restrict__ partial, int nparts, f
         if (int(threadIdx.x) < w) red[threadIdx.x] += red[threadIdx.x + w];
         __syncthreads();
     }
-    if (threadIdx.x == 0) *out = float(red[0] * double(scale));
-}
-
-// Advances the device step counter of a training run (last node of a step).
-__global__ void step_inc_kernel(int *step)
-{
-    pdl_wait();
-    pdl_trigger();
-    *step += 1;
-}
-
-// Adam on FP32 master parameters; refreshes the bf16 weight copies, the
-// tap-flipped transposed copies used by the backward pass, and the f32 biases.
-constexpr int kAdamLayers = 8;  // layers whose bf16 copies the Adam pass refreshes itself
-struct AdamArgs {
-    float *param, *m, *v;
-    const float *grad;
-    int64_t n;
-    float lr, b1, b2, eps, c1, c2;  // c1 = 1/(1-b1^t), c2 = 1/(1-b2^t)
-    // training runs: lr, c1, c2 of step *step from device arrays (null: the scalars above)
-    const int *step;
-    const float *lr_arr, *c1_arr, *c2_arr;
-    // bf16 copies written in the same pass (nl = 0: none): layer l's W[co][j][ci]
-    // at woff[l] (cout[l] x 5 x cin[l]) into w16 and, tap-flipped and
-    // transposed, into wt16 at the same offset (both in staging order)
-    bf16 *w16, *wt16;
-    int nl;
-    int64_t woff[kAdamLayers];
-    int cout[kAdamLayers], cin[kAdamLayers];
-};
-__global__ void adam_kernel(AdamArgs a)
-{
-    pdl_wait();
-    pdl_trigger();
-    const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (i >= a.n) return;
-    const float g = a.grad[i];
-    const float m = a.b1 * a.m[i] + (1.f - a.b1) * g;
-    const float v = a.b2 * a.v[i] + (1.f - a.b2) * g * g;
-    a.m[i] = m;
-    a.v[i] = v;
-    float lr = a.lr, c1 = a.c1, c2 = a.c2;
-    if (a.step) {
-        const int t = *a.step;
-        lr = a.lr_arr[t];
-        c1 = a.c1_arr[t];
-        c2 = a.c2_arr[t];
+    if (threadIdx.x == 0) {
+        if (losses) losses[*step] = float(red[0] * double(scale));
+        *step += 1;
     }
-    const float p = a.param[i] - lr * (m * c1) / (sqrtf(v * c2) + a.eps);
-    a.param[i] = p;
-    for (int l = 0; l < a.nl; ++l) {
-        const int64_t e = i - a.woff[l];
-        const int ci_ = a.cin[l], cout_ = a.cout[l];
-        if (e >= 0 && e < int64_t(cout_) * kTaps * ci_) {
-            const int co = int(e / (kTaps * ci_)), j = int((e / ci_) % kTaps), ci = int(e % ci_);
-            const bf16 b = __float2bfloat16(p);
-            a.w16[a.woff[l] + wstage_index(co, j, ci, cout_, ci_)] = b;
-            a.wt16[a.woff[l] + wstage_index(ci, kTaps - 1 - j, co, ci_, cout_)] = b;
-            break;
+}
+
+// The whole network on samples of up to kChainX positions, one CTA per sample:
+// input packing, every forward layer and the output (TRAIN = false), or also the
+// loss and the backward-data convolutions (TRAIN), which leaves the layer inputs
+// act[l] and the gradients dz[l] that the weight gradients read.
+//
+// One kernel per layer (conv_kernel) takes 6.7 items per SM through ramp, pipeline
+// fill and tail (10 to 12 us per 64-channel layer, 2.8 us at the tensor cores' rate),
+// and the edge terms, packing, loss and output passes were launches of their own.
+// 256 samples of 512 positions: forward 51.6 -> 26.9 us; with the backward pass 62 us, where
+// the launches took about 130.  Longer samples and deeper networks take the kernels
+// per layer.
+// Here a sample's activations (64 channels, 66 KB) stay in shared memory, overwritten
+// in place layer by layer: the products of all its 128-position tiles go to separate
+// TMEM accumulators (64 columns each), so the epilogue of tile i may overwrite the
+// tile once tile i + 1, which reads its last two positions, has its products.  The
+// arithmetic is conv_kernel's: same products in the same order, same bits.  Two CTAs
+// share an SM (one's products run beside the other's epilogue).
+constexpr int kChainX = 512;
+constexpr int kChainEpi = 8;  // epilogue warps: TMEM lane quarter w % 4, channel half w / 4
+constexpr int kChainThreads = 32 * (kChainEpi + 1);
+struct NetArgs {
+    struct {
+        int64_t woff, boff;
+        int cin, cout;  // padded
+        bf16 *act, *dz;  // input of the layer; gradient at its pre-activation (TRAIN)
+    } L[kChainLayers];
+    int nl, X, cin, cout;  // cin, cout: real channels of the network
+    const float *x, *y;    // [.][X][cin], [.][X][cout] (y: TRAIN)
+    const int32_t *per;
+    const int32_t *perm;  // mini-batch perm[*step B ..] of n samples; null: samples 0 .. B - 1
+    const int *step;
+    int64_t n;
+    const float *param, *norm;
+    const bf16 *w16, *wt16;
+    int32_t *perb;  // gathered padding kinds (perm)
+    float *out;     // prediction in physical units (TRAIN = false)
+    float grad_scale;
+    float *loss_partial;  // [B] sums of the squared error
+    unsigned *err;
+};
+inline size_t chain_smem(int X)
+{
+    const int rows = (X + kConvM - 1) / kConvM * kConvM + kTaps - 1;
+    return 16 * (size_t(kTaps) * 8 * 64 + size_t(8) * rows);
+}
+
+// The products of one layer for every tile, tile i's completion on tfull[i].
+template <int CIN, int COUT>
+__device__ __forceinline__ void chain_products(uint32_t taddr, uint32_t win, uint32_t ws, uint32_t alo, int tiles,
+                                               uint64_t *tfull, int leader)
+{
+    constexpr int KC = CIN / 8;
+    constexpr uint32_t BLBO = COUT * 16;
+    // descriptors move by their address field (16-byte units, no carry out of it)
+    const uint64_t db = umma_desc(ws, BLBO, 128);
+    uint64_t da = umma_desc(win, alo, 128);
+    for (int i = 0; i < tiles; ++i, da += kConvM) {
+        int step = 0;
+#pragma unroll
+        for (int j = 0; j < kTaps; ++j)
+#pragma unroll
+            for (int kc = 0; kc < KC; kc += 2, ++step)
+                umma_bf16_leader(taddr + i * 64, da + (uint32_t(kc) * (alo >> 4) + j),
+                                 db + (uint32_t(j * KC + kc) * (BLBO >> 4)), umma_idesc_bf16(kConvM, COUT), step, leader);
+        if (leader) umma_commit(&tfull[i]);
+        __syncwarp();
+    }
+}
+
+// 32 channels of a position as bf16, into rows c0 / 8 .. of the staged window and of a chunk-major tensor.
+template <int N>
+__device__ __forceinline__ void pack_row(const float (&v)[N], uint4 (&pk)[N / 8])
+{
+#pragma unroll
+    for (int q = 0; q < N / 8; ++q) {
+        __nv_bfloat162 *pp = reinterpret_cast<__nv_bfloat162 *>(&pk[q]);
+#pragma unroll
+        for (int h = 0; h < 4; ++h) pp[h] = __floats2bfloat162_rn(v[8 * q + 2 * h], v[8 * q + 2 * h + 1]);
+    }
+}
+
+template <bool TRAIN>
+__global__ void __launch_bounds__(kChainThreads, 2) net_kernel(const __grid_constant__ NetArgs a)
+{
+    constexpr int kTiles = kChainX / kConvM, ET = 32 * kChainEpi;
+    extern __shared__ __align__(128) unsigned char smem[];
+    bf16 *const ws = reinterpret_cast<bf16 *>(smem);  // weights of one layer, at most [40][64][8]
+    bf16 *const win = ws + kTaps * 8 * 64 * 8;        // [chunk][rows][8], row = position + 2
+    __shared__ __align__(8) uint64_t tfull[kTiles], wbar, ready, edged, done;
+    __shared__ __align__(16) float s_bias[kChainLayers][64], s_edge[2][64];
+    __shared__ float s_red[4];
+    __shared__ uint32_t s_taddr;
+    __shared__ int s_abort;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int X = a.X, nl = a.nl, tiles = (X + kConvM - 1) / kConvM, rows = tiles * kConvM + kTaps - 1;
+    const int last = tiles - 1, b = blockIdx.x;
+    const uint32_t ncol = tiles == 1 ? 64 : (tiles == 2 ? 128 : 256);
+    if (t == 0) {
+        for (int i = 0; i < kTiles; ++i) mbar_init(&tfull[i], 1);
+        mbar_init(&wbar, 1);
+        mbar_init(&done, 1);
+        mbar_init(&ready, ET);
+        mbar_init(&edged, ET);
+        s_abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == kChainEpi) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_taddr)),
+                     "r"(ncol)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    pdl_wait();
+    if (t == 0) pdl_trigger();
+    const uint32_t taddr = s_taddr;
+    volatile int *const abort = &s_abort;
+    // passes: forward layers 0 .. nl - 1, then (TRAIN) transposed layers nl - 1 .. 1
+    const int npass = TRAIN ? 2 * nl - 1 : nl;
+    if (warp == kChainEpi) {
+        {
+            const int leader = elect_one();
+            const uint32_t wa = smem_u32(win), wb = smem_u32(ws), alo = uint32_t(rows) * 16;
+            bool loading = false, ok = true;  // loading: a weight copy not yet waited for
+            uint32_t wparity = 0;
+            for (int p = 0; p < npass && ok; ++p) {
+                const bool bwd = p >= nl;
+                const auto &L = a.L[bwd ? 2 * nl - 1 - p : p];
+                const int ci = bwd ? L.cout : L.cin, co = bwd ? L.cin : L.cout;
+                // the weights, once the previous pass has read its own (products; the end terms)
+                if (p > 0) ok = __all_sync(0xffffffffu, mbar_wait(&tfull[last], (p - 1) & 1, abort));
+                if (ok && p > nl) ok = __all_sync(0xffffffffu, mbar_wait(&edged, (p - 1 - nl) & 1, abort));
+                if (!ok) break;
+                const uint32_t wbytes = uint32_t(kTaps) * ci * co * 2;
+                if (leader) {
+                    mbar_arrive_tx(&wbar, wbytes);
+                    bulk_g2s(ws, (bwd ? a.wt16 : a.w16) + L.woff, wbytes, &wbar);
+                }
+                __syncwarp();
+                loading = true;
+                wparity = p & 1;
+                ok = __all_sync(0xffffffffu, mbar_wait(&wbar, wparity, abort));
+                if (!ok) break;
+                loading = false;
+                ok = __all_sync(0xffffffffu, mbar_wait(&ready, p & 1, abort));
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                if (ci == 16) chain_products<16, 64>(taddr, wa, wb, alo, tiles, tfull, leader);
+                else if (co == 16) chain_products<64, 16>(taddr, wa, wb, alo, tiles, tfull, leader);
+                else chain_products<64, 64>(taddr, wa, wb, alo, tiles, tfull, leader);
+            }
+            // no copy and no product lands after the CTA has ended
+            if (leader) umma_commit(&done);
+            __syncwarp();
+            if (!mbar_wait(&done, 0, nullptr)) ok = false;
+            if (loading) mbar_wait(&wbar, wparity, nullptr);
+            if (!ok) give_up(abort, a.err);
         }
+        __syncwarp();
+    } else {
+        int64_t k = b;  // sample of this CTA
+        if (a.perm) {
+            k = a.perm[int64_t(*a.step) * gridDim.x + b];
+            if (k < 0 || k >= a.n) {
+                if (t == 0) atomicOr(a.err, 1u);
+                k = 0;
+            }
+        }
+        const int periodic = a.per[k];
+        if (a.perm && t == 0) a.perb[b] = periodic;
+        // The window is complete: its two rows before and after the sample (mode), then the
+        // tensor cores may read it.
+        auto publish = [&](int kc, int mode) {
+            asm volatile("bar.sync 1, %0;" ::"n"(ET) : "memory");
+            if (warp == 0)
+                for (int e = lane; e < 4 * kc; e += 32) {
+                    const int r = e & 3, c = e >> 2, row = r < 2 ? r : X + r;
+                    bool inside;
+                    const int src = wrap_pos(row - 2, X, mode, &inside) + 2;
+                    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+                    if (inside) v = *reinterpret_cast<const uint4 *>(win + (c * rows + src) * 8);
+                    *reinterpret_cast<uint4 *>(win + (c * rows + row) * 8) = v;
+                }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            mbar_arrive(&ready);
+        };
+        const int fmode = periodic != 0 ? PAD_PERIODIC : PAD_REPLICATE;
+        const int bmode = periodic != 0 ? PAD_PERIODIC : PAD_ZERO;
+        // input: the sample's features normalised
+        for (int p = t; p < X; p += ET) {
+            float v[kInPad];
+#pragma unroll
+            for (int c = 0; c < kInPad; ++c)
+                v[c] = c < 8 && c < a.cin ? (a.x[(k * X + p) * a.cin + c] - a.norm[c & 7]) * a.norm[8 + (c & 7)] : 0.f;
+            uint4 pk[2];
+            pack_row(v, pk);
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                *reinterpret_cast<uint4 *>(win + (q * rows + p + 2) * 8) = pk[q];
+                if (TRAIN) *reinterpret_cast<uint4 *>(a.L[0].act + cm_index(b, p, 8 * q, kInPad, X, 8)) = pk[q];
+            }
+        }
+        for (int e = t; e < nl * 64; e += ET) {
+            const int l = e >> 6, c = e & 63;
+            s_bias[l][c] = c < a.L[l].cout ? a.param[a.L[l].boff + c] : 0.f;
+        }
+        publish(kInPad / 8, fmode);
+
+        const int m = 32 * (warp & 3) + lane, c0 = 32 * (warp >> 2);  // position of a tile, first channel
+        const uint32_t tld = taddr + (uint32_t(32 * (warp & 3)) << 16);
+        bool ok = true;
+        uint32_t mask[(kChainLayers - 1) * kTiles];  // bit q of [l][i]: channel c0 + q of hidden layer l is > 0
+        // hidden layers; each tile's accumulator is read while the tile before is packed and stored
+        uint32_t r[32];
+        auto read_acc = [&](int i) {
+            tmem_ld16(r, tld + i * 64 + c0);
+            tmem_ld16(r + 16, tld + i * 64 + c0 + 16);
+        };
+        for (int l = 0; l < nl - 1; ++l) {
+            ok = mbar_wait(&tfull[0], l & 1, abort) && ok;
+            __syncwarp();
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            read_acc(0);
+            bf16 *o = TRAIN ? a.L[l + 1].act + cm_index(b, m, c0, 64, X, 8) : nullptr;
+            bf16 *so = win + ((c0 / 8) * rows + m + 2) * 8;
+#pragma unroll 1
+            for (int i = 0; i < tiles; ++i, o += kConvM * 8, so += kConvM * 8) {
+                // the products of the next tile, which read this tile's last positions
+                if (i < last) {
+                    ok = mbar_wait(&tfull[i + 1], l & 1, abort) && ok;
+                    __syncwarp();
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                }
+                tmem_wait(r);
+                float v[32];
+#pragma unroll
+                for (int q = 0; q < 32; q += 4) {
+                    const float4 bb = *reinterpret_cast<const float4 *>(&s_bias[l][c0 + q]);
+                    v[q] = fmaxf(__uint_as_float(r[q]) + bb.x, 0.f);
+                    v[q + 1] = fmaxf(__uint_as_float(r[q + 1]) + bb.y, 0.f);
+                    v[q + 2] = fmaxf(__uint_as_float(r[q + 2]) + bb.z, 0.f);
+                    v[q + 3] = fmaxf(__uint_as_float(r[q + 3]) + bb.w, 0.f);
+                }
+                uint4 pk[4];
+                pack_row(v, pk);
+                if (i < last) read_acc(i + 1);
+                if (TRAIN) {
+                    uint32_t mk = 0;
+                    const uint32_t *h = reinterpret_cast<const uint32_t *>(pk);
+#pragma unroll
+                    for (int q = 0; q < 16; ++q)
+                        mk |= ((h[q] & 0x7FFFu) ? 1u << (2 * q) : 0u) | ((h[q] & 0x7FFF0000u) ? 2u << (2 * q) : 0u);
+                    mask[l * kTiles + i] = mk;
+                }
+                if (i * kConvM + m < X) {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        *reinterpret_cast<uint4 *>(so + q * rows * 8) = pk[q];
+                        if (TRAIN) *reinterpret_cast<uint4 *>(o + int64_t(q) * X * 8) = pk[q];
+                    }
+                }
+                __syncwarp();
+            }
+            publish(8, fmode);
+        }
+        // output layer: prediction, or the squared error and its gradient
+        float se = 0.f;
+#pragma unroll 1
+        for (int i = 0; i < tiles; ++i) {
+            ok = mbar_wait(&tfull[i < last ? i + 1 : last], (nl - 1) & 1, abort) && ok;
+            __syncwarp();
+            if (warp >= 4) continue;  // 16 channels
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            uint32_t r[16];
+            tmem_ld16(r, tld + i * 64);
+            tmem_wait(r);
+            const int x = i * kConvM + m;
+            if (x >= X) continue;
+            if constexpr (!TRAIN) {
+#pragma unroll
+                for (int c = 0; c < 8; ++c)
+                    if (c < a.cout)
+                        a.out[(int64_t(b) * X + x) * a.cout + c] =
+                            (__uint_as_float(r[c]) + s_bias[nl - 1][c]) * a.norm[16 + c];
+            } else {
+                float g[16];
+#pragma unroll
+                for (int c = 0; c < 16; ++c) {
+                    float d = 0.f;
+                    if (c < 8 && c < a.cout) {
+                        d = (__uint_as_float(r[c]) + s_bias[nl - 1][c]) -
+                            a.y[(k * X + x) * a.cout + c] * a.norm[24 + (c & 7)];
+                        se += d * d;
+                    }
+                    g[c] = a.grad_scale * d;
+                }
+                uint4 pk[2];
+                pack_row(g, pk);
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    *reinterpret_cast<uint4 *>(win + (q * rows + x + 2) * 8) = pk[q];
+                    *reinterpret_cast<uint4 *>(a.L[nl - 1].dz + cm_index(b, x, 8 * q, kOutPad, X, 8)) = pk[q];
+                }
+            }
+        }
+        if constexpr (TRAIN) {
+            // the sample's squared error: lanes by shuffles, then the four warps in turn
+            if (warp < 4) {
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) se += __shfl_xor_sync(0xffffffffu, se, o);
+                if (lane == 0) s_red[warp] = se;
+            }
+            publish(kOutPad / 8, bmode);
+            if (t == 0) a.loss_partial[b] = ((s_red[0] + s_red[1]) + s_red[2]) + s_red[3];
+            // dz[l - 1] = (W^T * dz[l] + end terms of replicate padding) masked by act[l] > 0
+            for (int l = nl - 1; l > 0; --l) {
+                const int p = 2 * nl - 1 - l, co_n = a.L[l].cout;
+                ok = mbar_wait(&wbar, p & 1, abort) && ok;
+                // end terms (the sums of edge_grad_kernel, from the transposed weights of this pass)
+                if (t < 128 && periodic == 0) {
+                    const int side = t >> 6, ci = t & 63;
+                    const int ra = side ? 1 : 4, rb = side ? 0 : 3, rn = side ? 0 : 4;  // taps, flipped
+                    const int p0 = (side ? X - 1 : 0) + 2, p1 = (side ? X - 2 : 1) + 2;
+                    float acc = 0.f;
+                    for (int q = 0; q < co_n / 8; ++q) {
+                        auto row = [](const bf16 *p, float *f) {
+                            const uint4 u = *reinterpret_cast<const uint4 *>(p);
+                            const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&u);
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) {
+                                f[2 * k] = __bfloat162float(h[k].x);
+                                f[2 * k + 1] = __bfloat162float(h[k].y);
+                            }
+                        };
+                        float wa[8], wb[8], wn[8], d0[8], d1[8];
+                        row(ws + ((ra * (co_n / 8) + q) * 64 + ci) * 8, wa);
+                        row(ws + ((rb * (co_n / 8) + q) * 64 + ci) * 8, wb);
+                        row(ws + ((rn * (co_n / 8) + q) * 64 + ci) * 8, wn);
+                        row(win + (q * rows + p0) * 8, d0);
+                        row(win + (q * rows + p1) * 8, d1);
+#pragma unroll
+                        for (int h = 0; h < 8; ++h) {
+                            acc = fmaf(wa[h] + wb[h], d0[h], acc);
+                            acc = fmaf(wn[h], d1[h], acc);
+                        }
+                    }
+                    s_edge[side][ci] = acc;
+                }
+                mbar_arrive(&edged);
+                asm volatile("bar.sync 1, %0;" ::"n"(ET) : "memory");
+                ok = mbar_wait(&tfull[0], p & 1, abort) && ok;
+                __syncwarp();
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                read_acc(0);
+                bf16 *o = a.L[l - 1].dz + cm_index(b, m, c0, 64, X, 8);
+                bf16 *so = win + ((c0 / 8) * rows + m + 2) * 8;
+#pragma unroll 1
+                for (int i = 0; i < tiles; ++i, o += kConvM * 8, so += kConvM * 8) {
+                    if (i < last) {
+                        ok = mbar_wait(&tfull[i + 1], p & 1, abort) && ok;
+                        __syncwarp();
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    }
+                    const uint32_t mk = mask[(l - 1) * kTiles + i];
+                    tmem_wait(r);
+                    const int x = i * kConvM + m;
+                    float v[32];
+#pragma unroll
+                    for (int q = 0; q < 32; ++q) v[q] = __uint_as_float(r[q]);
+                    if (periodic == 0 && (x == 0 || x == X - 1)) {
+#pragma unroll
+                        for (int q = 0; q < 32; ++q) v[q] += s_edge[x != 0][c0 + q];
+                    }
+#pragma unroll
+                    for (int q = 0; q < 32; ++q) v[q] = (mk >> q) & 1u ? v[q] : 0.f;
+                    uint4 pk[4];
+                    pack_row(v, pk);
+                    __syncwarp();
+                    if (i < last) read_acc(i + 1);
+                    if (x < X) {
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            if (l > 1) *reinterpret_cast<uint4 *>(so + q * rows * 8) = pk[q];
+                            *reinterpret_cast<uint4 *>(o + int64_t(q) * X * 8) = pk[q];
+                        }
+                    }
+                    __syncwarp();
+                }
+                if (l > 1) publish(8, bmode);
+            }
+        }
+        if (!ok) give_up(abort, a.err);
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == kChainEpi) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncol) : "memory");
     }
 }
 
@@ -1117,36 +1712,53 @@ cudaError_t conv_any(int cin, int cout, int epi, const bf16 *in, const bf16 *w, 
     return cudaErrorInvalidValue;
 }
 
-// The weight-gradient grid: CTAs per SM by shared memory and by the TMEM
-// columns of their five accumulators, at most 2 (the partial buffer holds
-// 2 x SMs parts); *parts receives the grid, the number of partials to sum.
-template <int CIN, int COUT>
-cudaError_t wgrad_launch(const bf16 *dz, const bf16 *in, const int *per, int B, int X, int sms, float *partial,
-                         unsigned *err, int *parts, cudaStream_t s)
+// Whether the whole-network kernel takes the network.
+inline bool chain_supported(int nl, int X) { return nl <= kChainLayers && X <= kChainX; }
+
+template <bool TRAIN>
+cudaError_t net_launch(const NetArgs &a, int B, cudaStream_t s)
 {
-    constexpr int RD = kConvM, RI = kConvM + kTaps - 1;
-    constexpr size_t smem = size_t(kWgradStages) * 16 * (size_t(COUT / 8) * RD + size_t(CIN / 8) * RI);
-    constexpr int ntot = kTaps * (COUT == 64 ? CIN : COUT);
-    constexpr int ncol = ntot <= 32 ? 32 : (ntot <= 64 ? 64 : (ntot <= 128 ? 128 : (ntot <= 256 ? 256 : 512)));
-    auto k = wgrad_kernel<CIN, COUT>;
-    constexpr int threads = role_threads(kWgradEpiWarps);
-    static ShapeCache cache;
-    int per_sm = 0, dev_sms = 0;
-    cudaError_t e = ctas_per_sm(k, threads, smem, ncol, 2, cache, &per_sm, &dev_sms);
+    static std::atomic<int> set[kMaxDevices];  // the shared-memory limit, once per device
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    const int ntiles = B * ((X + kConvM - 1) / kConvM);
-    const int grid = std::max(1, std::min(ntiles, std::max(1, sms) * per_sm));
-    *parts = grid;
-    return launch(k, dim3(grid), dim3(threads), smem, s, dz, in, per, X, ntiles, partial, err);
+    auto k = net_kernel<TRAIN>;
+    if (dev < 0 || dev >= kMaxDevices || !set[dev].load()) {
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(chain_smem(kChainX)));
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                     int(cudaSharedmemCarveoutMaxShared));
+        if (e != cudaSuccess) return e;
+        if (dev >= 0 && dev < kMaxDevices) set[dev].store(1);
+    }
+    return launch(k, dim3(unsigned(B)), dim3(kChainThreads), chain_smem(a.X), s, a);
 }
 
-cudaError_t wgrad_any(int cin, int cout, const bf16 *dz, const bf16 *in, const int *per, int B, int X, int sms,
-                      float *partial, unsigned *err, int *parts, cudaStream_t s)
+// Parts of a layer's items: one per SM for a 64 x 64 layer, two for the others.  The sums'
+// grouping follows from it, so it does not depend on how parts are dealt to CTAs.
+inline int wgrad_parts(int cin, int cout, int ntiles, int sms)
 {
-    if (cin == 16 && cout == 64) return wgrad_launch<16, 64>(dz, in, per, B, X, sms, partial, err, parts, s);
-    if (cin == 64 && cout == 64) return wgrad_launch<64, 64>(dz, in, per, B, X, sms, partial, err, parts, s);
-    if (cin == 64 && cout == 16) return wgrad_launch<64, 16>(dz, in, per, B, X, sms, partial, err, parts, s);
-    return cudaErrorInvalidValue;
+    return std::max(1, std::min(ntiles, cin == 64 && cout == 64 ? sms : 2 * sms));
+}
+
+// Weight gradients of layers l0 .. l0 + nl - 1 (entries set by the caller in the order the
+// pipeline takes them), one CTA per SM.
+cudaError_t wgrad_launch(WgradArgs &a, int sms, cudaStream_t s)
+{
+    constexpr size_t smem = size_t(kWgradStages) * kWgradStageBytes;
+    static std::atomic<int> set[kMaxDevices];  // the shared-memory limit, once per device
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kMaxDevices || !set[dev].load()) {
+        e = cudaFuncSetAttribute(wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+        if (e != cudaSuccess) return e;
+        if (dev >= 0 && dev < kMaxDevices) set[dev].store(1);
+    }
+    a.njobs = 0;
+    for (int k = 0; k < a.ne; ++k) a.njobs += a.E[k].njobs;
+    return launch(wgrad_kernel, dim3(unsigned(std::max(1, std::min(sms, a.njobs)))),
+                  dim3(kWgradThreads), smem, s, a);
 }
 
 }  // namespace
@@ -1166,10 +1778,7 @@ struct ql_closure {
     std::vector<bf16 *> act;  // act[0] input (bf16), act[l] output of layer l (l < L)
     float *pred = nullptr;    // last layer output f32 [B][X][16]
     std::vector<bf16 *> dz;   // dz[l]: gradient wrt pre-activation of layer l (1-based), stored bf16
-    float *partial = nullptr;  // two halves of 2 x sms weight-gradient partials each
-    // a second stream for the end terms and partial sums of the backward pass, and its events
-    cudaStream_t side = nullptr;
-    std::vector<cudaEvent_t> events;
+    float *partial = nullptr;  // weight-gradient partials
     float *loss_partial = nullptr;
     float *edge = nullptr;  // [max_batch][2][64] end-position gradient terms of replicate padding
     float *norm = nullptr;  // in_shift[8], in_inv_scale[8], out_scale[8], inv_out_scale[8]
@@ -1185,7 +1794,7 @@ struct ql_closure {
     int *d_step = nullptr;
     float *d_sched = nullptr;
     int64_t sched_cap = 0;
-    int sms = 0;  // SMs of the device; the weight-gradient partial buffer holds 2 x sms parts
+    int sms = 0;  // SMs of the device
     int64_t step = 0;
     std::string err;
 };
@@ -1220,8 +1829,6 @@ static void closure_release(ql_closure *c)
         cfree_dev(c, p);
     if (c->gexec) cudaGraphExecDestroy(c->gexec);
     if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
-    for (cudaEvent_t e : c->events) cudaEventDestroy(e);
-    if (c->side) cudaStreamDestroy(c->side);
     for (bf16 *p : c->act) cfree_dev(c, p);
     for (bf16 *p : c->dz) cfree_dev(c, p);
 }
@@ -1290,74 +1897,136 @@ static ql_status check_flags(ql_closure *c)
 static ql_status enqueue_train_step(ql_closure *c, const float *x, const float *y, const int32_t *periodic,
                                     int64_t n, const int32_t *perm, int64_t B, float *losses);
 
-// Loss, gradients of all parameters into c->grad; loss (host) if not null.
-static ql_status backward(ql_closure *c, const float *y, const int32_t *yidx, const int *ystep, const int *per, int B,
-                          float *loss, float *losses = nullptr)
+// The whole-network kernel's arguments that do not depend on the batch.
+static NetArgs net_args(ql_closure *c)
+{
+    NetArgs a = {};
+    a.nl = int(c->layers.size());
+    for (int l = 0; l < a.nl; ++l) {
+        const Layer &L = c->layers[size_t(l)];
+        a.L[l].woff = L.woff;
+        a.L[l].boff = L.boff;
+        a.L[l].cin = L.cin;
+        a.L[l].cout = L.cout;
+        a.L[l].act = c->act[size_t(l)];
+        a.L[l].dz = c->dz[size_t(l)];
+    }
+    a.X = c->d.positions;
+    a.cin = c->d.in_channels;
+    a.cout = c->d.out_channels;
+    a.param = c->param;
+    a.norm = c->norm;
+    a.w16 = c->w16;
+    a.wt16 = c->wt16;
+    a.loss_partial = c->loss_partial;
+    a.err = c->bad;
+    return a;
+}
+
+// Mini-batch of a training run: samples perm[*step B ..] of n (perm null: samples 0 .. B - 1).
+struct BatchIndex {
+    const int32_t *perm = nullptr;
+    const int *step = nullptr;
+    int64_t n = 0;
+};
+
+// Forward pass, loss partials (their number in *nloss) and every layer's act and dz of a batch;
+// *per_batch: the batch's padding kinds.
+static ql_status propagate(ql_closure *c, const float *x, const float *y, const int32_t *per, const BatchIndex &ix,
+                           int B, int *nloss, const int32_t **per_batch)
 {
     const int X = c->d.positions, nl = int(c->layers.size());
     const int64_t npos = int64_t(B) * X;
-    const unsigned nb = mse_blocks(npos);
     const float gscale = 2.f / float(npos * c->d.out_channels);
-    QC_CUDA(c, launch(mse_kernel, dim3(nb), dim3(256), 0, c->stream, c->pred, y, yidx, ystep, X, npos,
+    *per_batch = ix.perm ? c->perb : per;
+    if (chain_supported(nl, X)) {
+        NetArgs a = net_args(c);
+        a.x = x;
+        a.y = y;
+        a.per = per;
+        a.perm = ix.perm;
+        a.step = ix.step;
+        a.n = ix.n;
+        a.perb = c->perb;
+        a.grad_scale = gscale;
+        *nloss = B;
+        QC_CUDA(c, net_launch<true>(a, B, c->stream));
+        return QL_OK;
+    }
+    ql_status st = QL_OK;
+    if (ix.perm) {
+        QC_CUDA(c, launch(pack_gather_kernel, dim3(unsigned((npos + 255) / 256)), dim3(256), 0, c->stream, x, per,
+                          ix.perm, ix.step, ix.n, B, X, c->d.in_channels, c->norm, c->norm + 8, c->act[0], c->perb,
+                          c->bad));
+    } else {
+        st = pack(c, x, B);
+    }
+    if (st == QL_OK) st = forward(c, *per_batch, B);
+    if (st != QL_OK) return st;
+    const unsigned nb = mse_blocks(npos);
+    *nloss = int(nb);
+    QC_CUDA(c, launch(mse_kernel, dim3(nb), dim3(256), 0, c->stream, c->pred, y, ix.perm, ix.step, ix.n, X, npos,
                       c->d.out_channels, c->norm + 24, gscale, c->dz[nl - 1], c->loss_partial));
-    // The weight gradients and backward-data convolutions run on c->stream; the end terms of
-    // layer l (after dz[l] is written) and the sum of layer l's weight-gradient partials (after
-    // they are written) run on a second stream beside them, joined by events: the end terms
-    // before the backward-data convolution that adds them, every partial sum before the end of
-    // the pass.  Layer l's partials sit in half l % 2 of the partial buffer, so that the next
-    // layer's weight gradient does not wait for this layer's sum.
-    // per layer l: [4 l] dz[l] ready, [4 l + 1] end terms, [4 l + 2] partials; [3] the join at the
-    // end, [4 (nl - 1) + 3] the loss partials
-    cudaEvent_t *ev = c->events.data();
-    const size_t half = size_t(2 * c->sms) * (64 * kTaps * 64 + 64);
-    if (losses) {
-        // a training run's per-step loss (device array, slot *ystep), on the second stream
-        QC_CUDA(c, cudaEventRecord(ev[4 * (nl - 1) + 3], c->stream));
-        QC_CUDA(c, cudaStreamWaitEvent(c->side, ev[4 * (nl - 1) + 3], 0));
-        QC_CUDA(c, launch(loss_sum_kernel, dim3(1), dim3(256), 0, c->side, c->loss_partial, int(nb),
-                          float(1.0 / double(npos * c->d.out_channels)), losses, ystep));
+    for (int l = nl - 1; l > 0; --l) {
+        // dz[l-1] = (W^T * dz[l] + end terms of replicate padding) masked by act[l] > 0
+        // (act[l] is the output of layer l-1)
+        const Layer &L = c->layers[size_t(l)];
+        static_assert(kEdgeSamples * kEdgeChannels == 256, "one output per thread");
+        QC_CUDA(c, launch(edge_grad_kernel,
+                          dim3((B + kEdgeSamples - 1) / kEdgeSamples, 2, (L.cin + kEdgeChannels - 1) / kEdgeChannels),
+                          dim3(256), 0, c->stream, c->dz[l], c->w16 + L.woff, *per_batch, B, X, L.cout, L.cin,
+                          c->edge));
+        QC_CUDA(c, conv_any(L.cout, L.cin, EPI_MASK_BF16, c->dz[l], c->wt16 + L.woff, nullptr, *per_batch, B, X,
+                            c->dz[l - 1], c->act[l], c->edge, c->bad, c->stream));
     }
-    for (int l = nl - 1; l >= 0; --l) {
-        const Layer &L = c->layers[l];
-        const int len = L.cout * kTaps * L.cin + L.cout;  // a multiple of 4 (channels are padded to 16)
-        if (len % 4 != 0) return cfail(c, QL_EUNSUPPORTED, "channel padding");
-        float *part = c->partial + (l % 2) * half;
-        if (l > 0) {
-            // end terms of replicate padding for dz[l-1], beside the weight gradient
-            static_assert(kEdgeSamples * kEdgeChannels == 256, "one output per thread");
-            QC_CUDA(c, cudaEventRecord(ev[4 * l], c->stream));
-            QC_CUDA(c, cudaStreamWaitEvent(c->side, ev[4 * l], 0));
-            QC_CUDA(c, launch(edge_grad_kernel,
-                              dim3((B + kEdgeSamples - 1) / kEdgeSamples, 2, (L.cin + kEdgeChannels - 1) / kEdgeChannels),
-                              dim3(256), 0, c->side, c->dz[l], c->w16 + L.woff, per, B, X, L.cout, L.cin, c->edge));
-            QC_CUDA(c, cudaEventRecord(ev[4 * l + 1], c->side));
+    return QL_OK;
+}
+
+// The gradients of all parameters from act and dz into c->grad, and (adam not null) the Adam
+// update with them; kChainLayers layers per launch.
+static ql_status weight_gradients(ql_closure *c, const int32_t *per, int B, const AdamArgs *adam)
+{
+    const int nl = int(c->layers.size());
+    for (int l0 = 0; l0 < nl; l0 += kChainLayers) {
+        const int ng = std::min(kChainLayers, nl - l0);
+        WgradArgs w = {};
+        w.periodic = per;
+        w.X = c->d.positions;
+        w.ntiles = B * ((w.X + kConvM - 1) / kConvM);
+        w.err = c->bad;
+        ReduceArgs r = {};
+        r.grad = c->grad;
+        float *partial = c->partial;
+        unsigned blocks = 0;
+        // 64 x 64 layers and halves of the others in turn (their accumulators differ)
+        WgradEntry big[kChainLayers], small[2 * kChainLayers];
+        int nbig = 0, nsmall = 0;
+        for (int l = 0; l < ng; ++l) {
+            const Layer &L = c->layers[size_t(l0 + l)];
+            WgradEntry e = {c->dz[size_t(l0 + l)], c->act[size_t(l0 + l)], partial, L.cin, L.cout, 0, 0, 0};
+            e.nparts = e.njobs = wgrad_parts(L.cin, L.cout, w.ntiles, c->sms);
+            r.L[l] = {partial, e.nparts, L.cout, L.cin, L.woff};
+            blocks = std::max(blocks, unsigned(reduce_blocks(L.cin, L.cout)));
+            partial += size_t(e.nparts) * wgrad_len(L.cin, L.cout);
+            if (L.cin == 64 && L.cout == 64) {
+                big[nbig++] = e;
+                continue;
+            }
+            WgradEntry e2 = e;
+            e.njobs = (e.nparts + 1) / 2;
+            e2.part0 = e.njobs;
+            e2.njobs = e.nparts - e.njobs;
+            small[nsmall++] = e;
+            small[nsmall++] = e2;
         }
-        int parts = 0;
-        QC_CUDA(c, wgrad_any(L.cin, L.cout, c->dz[l], c->act[l], per, B, X, c->sms, part, c->bad, &parts,
-                             c->stream));
-        // partial layout per CTA: [cout][5 cin] then [cout]; W and b are contiguous in the parameter vector
-        QC_CUDA(c, cudaEventRecord(ev[4 * l + 2], c->stream));
-        QC_CUDA(c, cudaStreamWaitEvent(c->side, ev[4 * l + 2], 0));
-        QC_CUDA(c, launch(reduce_partials_kernel, dim3((len + 127) / 128), dim3(32 * kReduceWarps), 0, c->side,
-                          part, parts, len, c->grad + L.woff));
-        if (l > 0) {
-            // dz[l-1] = (W^T * dz[l] + end terms of replicate padding) masked by act[l] > 0
-            // (act[l] is the output of layer l-1)
-            QC_CUDA(c, cudaStreamWaitEvent(c->stream, ev[4 * l + 1], 0));
-            QC_CUDA(c, conv_any(L.cout, L.cin, EPI_MASK_BF16, c->dz[l], c->wt16 + L.woff, nullptr, per, B, X,
-                                c->dz[l - 1], c->act[l], c->edge, c->bad, c->stream));
+        for (int k = 0; k < std::max(nbig, nsmall); ++k) {
+            if (k < nbig) w.E[w.ne++] = big[k];
+            if (k < nsmall) w.E[w.ne++] = small[k];
         }
-    }
-    // the side stream's last partial sum before anything that follows on c->stream
-    QC_CUDA(c, cudaEventRecord(ev[3], c->side));
-    QC_CUDA(c, cudaStreamWaitEvent(c->stream, ev[3], 0));
-    if (loss) {
-        std::vector<float> h(nb);
-        QC_CUDA(c, cudaMemcpyAsync(h.data(), c->loss_partial, sizeof(float) * nb, cudaMemcpyDeviceToHost, c->stream));
-        QC_CUDA(c, cudaStreamSynchronize(c->stream));
-        double s = 0;
-        for (float v : h) s += v;
-        *loss = float(s / double(npos * c->d.out_channels));
+        QC_CUDA(c, wgrad_launch(w, c->sms, c->stream));
+        const dim3 grid(blocks, unsigned(ng)), block(32 * kReduceWarps);
+        if (adam) QC_CUDA(c, launch(reduce_partials_kernel<true>, grid, block, 0, c->stream, r, *adam));
+        else QC_CUDA(c, launch(reduce_partials_kernel<false>, grid, block, 0, c->stream, r, AdamArgs{}));
     }
     return QL_OK;
 }
@@ -1416,12 +2085,19 @@ ql_status ql_closure_create(const ql_closure_desc *d, const ql_opts *opts, ql_cl
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
     c->sms = sms > 0 ? sms : 128;
-    c->partial = static_cast<float *>(calloc_dev(c, sizeof(float) * 2 * size_t(2 * c->sms) * (64 * kTaps * 64 + 64)));
-    if (cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess) c->side = nullptr;
-    c->events.assign(size_t(4 * d->layers), nullptr);
-    for (cudaEvent_t &e : c->events)
-        if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) e = nullptr;
-    c->loss_partial = static_cast<float *>(calloc_dev(c, sizeof(float) * mse_blocks(npos)));
+    size_t npartial = 0;  // of the largest group of layers a weight-gradient launch takes
+    for (int l0 = 0; l0 < d->layers; l0 += kChainLayers) {
+        size_t group = 0;
+        for (int l = l0; l < std::min(l0 + kChainLayers, int(d->layers)); ++l) {
+            const Layer &L = c->layers[size_t(l)];
+            group += size_t(wgrad_parts(L.cin, L.cout, B * ((X + kConvM - 1) / kConvM), c->sms)) *
+                     wgrad_len(L.cin, L.cout);
+        }
+        npartial = std::max(npartial, group);
+    }
+    c->partial = static_cast<float *>(calloc_dev(c, sizeof(float) * npartial));
+    c->loss_partial =
+        static_cast<float *>(calloc_dev(c, sizeof(float) * std::max(size_t(B), size_t(mse_blocks(npos)))));
     c->edge = static_cast<float *>(calloc_dev(c, sizeof(float) * size_t(B) * 2 * 64));
     c->perb = static_cast<int32_t *>(calloc_dev(c, sizeof(int32_t) * size_t(B)));
     c->bad = static_cast<unsigned *>(calloc_dev(c, sizeof(unsigned)));
@@ -1429,9 +2105,6 @@ ql_status ql_closure_create(const ql_closure_desc *d, const ql_opts *opts, ql_cl
               c->loss_partial && c->edge && c->perb && c->bad;
     for (int l = 0; l < d->layers; ++l) ok = ok && c->act[l] && c->dz[l];
     if (!ok) return bail(QL_ENOMEM, "closure allocation failed");
-    bool evok = c->side != nullptr;
-    for (cudaEvent_t e : c->events) evok = evok && e != nullptr;
-    if (!evok) return bail(QL_ECUDA, "closure stream or event creation failed");
 
     // seeded He-uniform weights (real channels only), zero biases and padding
     std::vector<float> h(off, 0.f);
@@ -1471,6 +2144,14 @@ ql_status ql_closure_create(const ql_closure_desc *d, const ql_opts *opts, ql_cl
 ql_status ql_closure_forward(ql_closure *c, const float *x, const int32_t *periodic, int64_t B, float *y)
 {
     if (!c || !x || !periodic || !y || B < 1 || B > c->d.max_batch) return cfail(c, QL_EINVAL, "bad arguments");
+    if (chain_supported(int(c->layers.size()), c->d.positions)) {
+        NetArgs a = net_args(c);
+        a.x = x;
+        a.per = periodic;
+        a.out = y;
+        QC_CUDA(c, net_launch<false>(a, int(B), c->stream));
+        return QL_OK;
+    }
     ql_status st = pack(c, x, int(B));
     if (st == QL_OK) st = forward(c, periodic, int(B));
     if (st != QL_OK) return st;
@@ -1485,10 +2166,20 @@ ql_status ql_closure_gradients(ql_closure *c, const float *x, const float *y, co
                                float *loss, float *grad_host)
 {
     if (!c || !x || !y || !periodic || B < 1 || B > c->d.max_batch) return cfail(c, QL_EINVAL, "bad arguments");
-    ql_status st = pack(c, x, int(B));
-    if (st == QL_OK) st = forward(c, periodic, int(B));
-    if (st == QL_OK) st = backward(c, y, nullptr, nullptr, periodic, int(B), loss);
+    int nloss = 0;
+    const int32_t *per = nullptr;
+    ql_status st = propagate(c, x, y, periodic, BatchIndex(), int(B), &nloss, &per);
+    if (st == QL_OK) st = weight_gradients(c, per, int(B), nullptr);
     if (st != QL_OK) return st;
+    if (loss) {
+        std::vector<float> h(static_cast<size_t>(nloss));
+        QC_CUDA(c, cudaMemcpyAsync(h.data(), c->loss_partial, sizeof(float) * h.size(), cudaMemcpyDeviceToHost,
+                                   c->stream));
+        QC_CUDA(c, cudaStreamSynchronize(c->stream));
+        double s = 0;
+        for (float v : h) s += v;
+        *loss = float(s / double(B * c->d.positions * c->d.out_channels));
+    }
     if (grad_host) {
         QC_CUDA(c, cudaMemcpyAsync(grad_host, c->grad, sizeof(float) * c->nparam, cudaMemcpyDeviceToHost, c->stream));
         QC_CUDA(c, cudaStreamSynchronize(c->stream));
@@ -1621,24 +2312,23 @@ static AdamArgs adam_args(ql_closure *c)
 static ql_status enqueue_train_step(ql_closure *c, const float *x, const float *y, const int32_t *periodic,
                                     int64_t n, const int32_t *perm, int64_t B, float *losses)
 {
-    const int X = c->d.positions;
-    QC_CUDA(c, launch(pack_gather_kernel, dim3(unsigned((B * X + 255) / 256)), dim3(256), 0, c->stream, x, periodic,
-                      perm, c->d_step, n, int(B), X, c->d.in_channels, c->norm, c->norm + 8, c->act[0], c->perb,
-                      c->bad));
-    ql_status st = forward(c, c->perb, int(B));
-    if (st == QL_OK) st = backward(c, y, perm, c->d_step, c->perb, int(B), nullptr, losses);
-    if (st != QL_OK) return st;
+    BatchIndex ix;
+    ix.perm = perm;
+    ix.step = c->d_step;
+    ix.n = n;
+    int nloss = 0;
+    const int32_t *per = nullptr;
     AdamArgs a = adam_args(c);
     a.step = c->d_step;
     a.lr_arr = c->d_sched;
     a.c1_arr = c->d_sched + c->sched_cap;
     a.c2_arr = c->d_sched + 2 * c->sched_cap;
-    QC_CUDA(c, launch(adam_kernel, dim3(unsigned((c->nparam + 255) / 256)), dim3(256), 0, c->stream, a));
-    if (!a.nl) {
-        st = refresh_weights(c);
-        if (st != QL_OK) return st;
-    }
-    QC_CUDA(c, launch(step_inc_kernel, dim3(1), dim3(1), 0, c->stream, c->d_step));
+    ql_status st = propagate(c, x, y, periodic, ix, int(B), &nloss, &per);
+    if (st == QL_OK) st = weight_gradients(c, per, int(B), &a);
+    if (st == QL_OK && !a.nl) st = refresh_weights(c);
+    if (st != QL_OK) return st;
+    QC_CUDA(c, launch(loss_step_kernel, dim3(1), dim3(256), 0, c->stream, c->loss_partial, nloss,
+                      float(1.0 / double(B * c->d.positions * c->d.out_channels)), losses, c->d_step));
     return QL_OK;
 }
 
