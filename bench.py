@@ -683,7 +683,7 @@ def run_learned(args):
                        "batch": args.train_batch, "lr": args.lr, "lr_schedule": "cosine to lr/20"},
             # per training step (graph nodes): gather + pack, 5 convs, mse, 5 wgrads + 5 partial sums,
             # 4 edge terms + 4 transposed convs, loss sum, adam (with the weight casts), step counter
-            "gpu_launches": 28 * (nsamp // args.train_batch), "train_conv_tflops": train_tflops,
+            "gpu_launches": 4 * (nsamp // args.train_batch), "train_conv_tflops": train_tflops,
             "roofline": _tensor_roofline(train_tflops), "data_generation_s": t_gen,
             "train_s": t_train, "loss_per_epoch": losses, "held_out": held,
             "time_to_solution": {"pairs": n, "coarse_fp32_batch_plus_net_s": t_learned,

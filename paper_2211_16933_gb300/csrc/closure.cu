@@ -521,7 +521,7 @@ __global__ void __launch_bounds__(role_threads(conv_epi_warps(COUT)), 2)
 // [column j N + n][m], 64 consecutive bytes per warp and column, then the 64 or 16 bias sums;
 // reduce_partials_kernel sums the partials in a fixed order.  A wait that gives up sets bit
 // 1 of *err and ends the CTA's work.
-constexpr int kChainLayers = 8;  // layers of one launch (weight gradients, whole-network kernel)
+constexpr int kChainLayers = 8;  // layers of one weight-gradient launch
 struct WgradEntry {  // parts part0 .. part0 + njobs - 1 (of nparts) of a layer
     const bf16 *dz, *in;
     float *partial;  // [nparts][wgrad_len]
@@ -1189,24 +1189,28 @@ __global__ void loss_step_kernel(const float *__restrict__ partial, int nparts, 
 // One kernel per layer (conv_kernel) takes 6.7 items per SM through ramp, pipeline
 // fill and tail (10 to 12 us per 64-channel layer, 2.8 us at the tensor cores' rate),
 // and the edge terms, packing, loss and output passes were launches of their own.
-// 256 samples of 512 positions: forward 51.6 -> 26.9 us; with the backward pass 62 us, where
-// the launches took about 130.  Longer samples and deeper networks take the kernels
-// per layer.
+// 256 samples of 512 positions: forward 51.6 -> 25.9 us; with the backward pass 66 us, where
+// the launches took about 130.  Of these 66, the stores of act and dz (142 MB) cost 11; the
+// tensor pipe is busy 37 % of the time.  Longer samples (their activations do not fit) and
+// deeper networks take the kernels per layer.
 // Here a sample's activations (64 channels, 66 KB) stay in shared memory, overwritten
 // in place layer by layer: the products of all its 128-position tiles go to separate
 // TMEM accumulators (64 columns each), so the epilogue of tile i may overwrite the
 // tile once tile i + 1, which reads its last two positions, has its products.  The
 // arithmetic is conv_kernel's: same products in the same order, same bits.  Two CTAs
-// share an SM (one's products run beside the other's epilogue).
-constexpr int kChainX = 512;
-constexpr int kChainEpi = 8;  // epilogue warps: TMEM lane quarter w % 4, channel half w / 4
+// share an SM (one's products run beside the other's epilogue); 16 epilogue warps of 16 channels
+// each are 4 % faster than 8 of 32, and two samples in one CTA, their products in turn, 10 %
+// slower.
+constexpr int kChainX = 512, kNetLayers = 5;  // positions and layers it takes
+constexpr int kChainEpi = 16;  // epilogue warps: TMEM lane quarter w % 4, channel group w / 4
+constexpr int kChainNc = 64 / (kChainEpi / 4);  // channels of a group
 constexpr int kChainThreads = 32 * (kChainEpi + 1);
 struct NetArgs {
     struct {
         int64_t woff, boff;
         int cin, cout;  // padded
         bf16 *act, *dz;  // input of the layer; gradient at its pre-activation (TRAIN)
-    } L[kChainLayers];
+    } L[kNetLayers];
     int nl, X, cin, cout;  // cin, cout: real channels of the network
     const float *x, *y;    // [.][X][cin], [.][X][cout] (y: TRAIN)
     const int32_t *per;
@@ -1270,7 +1274,7 @@ __global__ void __launch_bounds__(kChainThreads, 2) net_kernel(const __grid_cons
     bf16 *const ws = reinterpret_cast<bf16 *>(smem);  // weights of one layer, at most [40][64][8]
     bf16 *const win = ws + kTaps * 8 * 64 * 8;        // [chunk][rows][8], row = position + 2
     __shared__ __align__(8) uint64_t tfull[kTiles], wbar, ready, edged, done;
-    __shared__ __align__(16) float s_bias[kChainLayers][64], s_edge[2][64];
+    __shared__ __align__(16) float s_bias[kNetLayers][64], s_edge[2][64];
     __shared__ float s_red[4];
     __shared__ uint32_t s_taddr;
     __shared__ int s_abort;
@@ -1392,15 +1396,29 @@ __global__ void __launch_bounds__(kChainThreads, 2) net_kernel(const __grid_cons
         }
         publish(kInPad / 8, fmode);
 
-        const int m = 32 * (warp & 3) + lane, c0 = 32 * (warp >> 2);  // position of a tile, first channel
+        constexpr int NC = kChainNc;
+        const int m = 32 * (warp & 3) + lane, c0 = NC * (warp >> 2);  // position of a tile, first channel
         const uint32_t tld = taddr + (uint32_t(32 * (warp & 3)) << 16);
         bool ok = true;
-        uint32_t mask[(kChainLayers - 1) * kTiles];  // bit q of [l][i]: channel c0 + q of hidden layer l is > 0
+        // Per tile a stack of 16 bits per hidden layer (bit q: channel c0 + q is > 0), pushed forward and
+        // popped backward; rotated so that the tile at hand is mask0 (an array indexed by the
+        // tile lies in local memory: 69 us per training step instead of 66).
+        static_assert(NC == 16 && 16 * (kNetLayers - 1) <= 64, "one 64-bit stack per tile");
+        uint64_t mask0 = 0, mask1 = 0, mask2 = 0, mask3 = 0;
+        auto next_mask = [&](uint64_t stack) {
+            mask0 = mask1;
+            mask1 = mask2;
+            mask2 = mask3;
+            mask3 = stack;
+        };
+        auto align_masks = [&] {  // after a loop over the tiles
+            for (int i = tiles; i < kTiles; ++i) next_mask(mask0);
+        };
         // hidden layers; each tile's accumulator is read while the tile before is packed and stored
-        uint32_t r[32];
+        uint32_t r[NC];
         auto read_acc = [&](int i) {
-            tmem_ld16(r, tld + i * 64 + c0);
-            tmem_ld16(r + 16, tld + i * 64 + c0 + 16);
+#pragma unroll
+            for (int q = 0; q < NC; q += 16) tmem_ld16(r + q, tld + i * 64 + c0 + q);
         };
         for (int l = 0; l < nl - 1; ++l) {
             ok = mbar_wait(&tfull[0], l & 1, abort) && ok;
@@ -1418,35 +1436,36 @@ __global__ void __launch_bounds__(kChainThreads, 2) net_kernel(const __grid_cons
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 }
                 tmem_wait(r);
-                float v[32];
+                float v[NC];
 #pragma unroll
-                for (int q = 0; q < 32; q += 4) {
+                for (int q = 0; q < NC; q += 4) {
                     const float4 bb = *reinterpret_cast<const float4 *>(&s_bias[l][c0 + q]);
                     v[q] = fmaxf(__uint_as_float(r[q]) + bb.x, 0.f);
                     v[q + 1] = fmaxf(__uint_as_float(r[q + 1]) + bb.y, 0.f);
                     v[q + 2] = fmaxf(__uint_as_float(r[q + 2]) + bb.z, 0.f);
                     v[q + 3] = fmaxf(__uint_as_float(r[q + 3]) + bb.w, 0.f);
                 }
-                uint4 pk[4];
+                uint4 pk[NC / 8];
                 pack_row(v, pk);
                 if (i < last) read_acc(i + 1);
                 if (TRAIN) {
                     uint32_t mk = 0;
                     const uint32_t *h = reinterpret_cast<const uint32_t *>(pk);
 #pragma unroll
-                    for (int q = 0; q < 16; ++q)
+                    for (int q = 0; q < NC / 2; ++q)
                         mk |= ((h[q] & 0x7FFFu) ? 1u << (2 * q) : 0u) | ((h[q] & 0x7FFF0000u) ? 2u << (2 * q) : 0u);
-                    mask[l * kTiles + i] = mk;
+                    next_mask(mask0 << 16 | mk);
                 }
                 if (i * kConvM + m < X) {
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
+                    for (int q = 0; q < NC / 8; ++q) {
                         *reinterpret_cast<uint4 *>(so + q * rows * 8) = pk[q];
                         if (TRAIN) *reinterpret_cast<uint4 *>(o + int64_t(q) * X * 8) = pk[q];
                     }
                 }
                 __syncwarp();
             }
+            if (TRAIN) align_masks();
             publish(8, fmode);
         }
         // output layer: prediction, or the squared error and its gradient
@@ -1547,31 +1566,33 @@ __global__ void __launch_bounds__(kChainThreads, 2) net_kernel(const __grid_cons
                         __syncwarp();
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     }
-                    const uint32_t mk = mask[(l - 1) * kTiles + i];
+                    const uint32_t mk = uint32_t(mask0) & 0xFFFFu;
+                    next_mask(mask0 >> 16);
                     tmem_wait(r);
                     const int x = i * kConvM + m;
-                    float v[32];
+                    float v[NC];
 #pragma unroll
-                    for (int q = 0; q < 32; ++q) v[q] = __uint_as_float(r[q]);
+                    for (int q = 0; q < NC; ++q) v[q] = __uint_as_float(r[q]);
                     if (periodic == 0 && (x == 0 || x == X - 1)) {
 #pragma unroll
-                        for (int q = 0; q < 32; ++q) v[q] += s_edge[x != 0][c0 + q];
+                        for (int q = 0; q < NC; ++q) v[q] += s_edge[x != 0][c0 + q];
                     }
 #pragma unroll
-                    for (int q = 0; q < 32; ++q) v[q] = (mk >> q) & 1u ? v[q] : 0.f;
-                    uint4 pk[4];
+                    for (int q = 0; q < NC; ++q) v[q] = (mk >> q) & 1u ? v[q] : 0.f;
+                    uint4 pk[NC / 8];
                     pack_row(v, pk);
                     __syncwarp();
                     if (i < last) read_acc(i + 1);
                     if (x < X) {
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) {
+                        for (int q = 0; q < NC / 8; ++q) {
                             if (l > 1) *reinterpret_cast<uint4 *>(so + q * rows * 8) = pk[q];
                             *reinterpret_cast<uint4 *>(o + int64_t(q) * X * 8) = pk[q];
                         }
                     }
                     __syncwarp();
                 }
+                align_masks();
                 if (l > 1) publish(8, bmode);
             }
         }
@@ -1713,7 +1734,7 @@ cudaError_t conv_any(int cin, int cout, int epi, const bf16 *in, const bf16 *w, 
 }
 
 // Whether the whole-network kernel takes the network.
-inline bool chain_supported(int nl, int X) { return nl <= kChainLayers && X <= kChainX; }
+inline bool chain_supported(int nl, int X) { return nl <= kNetLayers && X <= kChainX; }
 
 template <bool TRAIN>
 cudaError_t net_launch(const NetArgs &a, int B, cudaStream_t s)
