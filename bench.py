@@ -49,7 +49,7 @@ def _tensor_roofline(achieved_tflops):
         peak, src = 1700.0, "fallback (sustained)"
     return {"bound": "tensor", "achieved": achieved_tflops, "peak": peak, "unit": "TFLOP/s",
             "frac": achieved_tflops / peak, "traffic": None, "peak_source": src,
-            "kernel": "closure training step: conv_kernel, wgrad_kernel, transposed conv_kernel"}
+            "kernel": "closure training step: net_kernel, wgrad_kernel, reduce_partials_kernel, loss_step_kernel"}
 
 
 # Sources the stage kernels of each precision are compiled from (the unit and what it includes).
