@@ -130,7 +130,9 @@ __device__ __forceinline__ void weno5_faces_i64(const double (&a)[N], const doub
     for (int k = 0; k < N; ++k) {
         float rf;
         asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(float(uint32_t(S[k] >> 32))));
-        x0[k] = uint64_t(uint32_t(rf * 2305843009213693952.0f)) << 32;
+        // S = 2^62 (one weight, of indicators that are powers of two, outweighs the others) has X =
+        // 2^63, which as a signed number turns the correction round: x0 stays below it, and so does X
+        x0[k] = uint64_t(min(uint32_t(rf * 2305843009213693952.0f), 0x7FFFFFFFu)) << 32;
         d[k] = int64_t(0x2000000000000000ull - __umul64hi(S[k], x0[k]));
         const int32_t dd = int32_t(d[k] >> 10);
         d[k] += (int64_t(dd) * dd) >> 41;
