@@ -9,33 +9,41 @@
 // weighted sum in integers beside the FP64 pipe, and the result is added to f0
 // by one fused multiply-add.
 //
-// Fixed point: the four differences share the largest one's exponent, its
-// leading bit at bit 58, so each carries at least 6 bits more than its own
-// double and is cut at 2^-58 of the largest.  Each smoothness indicator is
-// normalised on its own (63 bits and an exponent), so that small indicators keep
-// their relative precision: a small stencil's weight error only multiplies
-// that stencil's equally small candidate.  Weights and their sum are normalised to
-// 62 bits, the quotient comes from a reciprocal refined by one third-order
-// step.  The total error is below 2^-55 of the largest difference, under the
-// rounding of the final addition: against quadruple precision the largest error
-// over rough, smooth, jump and flat data is 0.60 of that of the FP64 form it
-// replaces, and never larger.
+// Fixed point: the two differences of each stencil share the larger one's exponent, its
+// leading bit at bit 59, so each carries at least 7 bits more than its own
+// double and is cut at 2^-59 of the stencil's larger one.  Each smoothness indicator is
+// normalised on its own (63 bits and an exponent).  The weighted sum is formed in the unit of its
+// largest term: a stencil's differences may be 2^k times the smoothest one's, its weight is then about
+// 2^-4k of it, so that it stays within a few bits of the smoothest one's unit.  The error is about 2^-54 of the
+// differences of the stencils that carry the weight, whatever the other differences are: values far
+// smaller than a jump beside them (populations of fast velocities at an unresolved jump) keep their relative
+// precision and their sign.  (One exponent for all four differences, the former form, made +-5e-18 of a tail of
+// 1e-25 beside a value of 1.)  Weights and their sum are normalised to 62 bits, the
+// quotient comes from a reciprocal refined by one third-order step.
+// Against quadruple precision, largest and mean error over max(|f0|, |h|) in units of 1e-16, FP64 product form -> this
+// (4e6 faces each, the largest difference between a half and twice f0): random data 4.95, 0.402 -> 1.69, 0.370;
+// Gaussian profiles 2.29, 0.407 -> 1.65, 0.370; a jump between nearly flat sides 1.42, 0.398 -> 1.18, 0.398; values
+// falling by e^5 per cell 3.49, 0.678 -> 1.64, 0.404, rising by e^12 2.68, 0.527 -> 1.82, 0.494; a tail of 1e-25
+// beside 1 1.24, 0.461 -> 1.27, 0.460; exponents uniform in e^+-8 4970, 1.03 -> 3310, 0.778.  The exponents per stencil
+// cost the tile kernels 3 % (262144 cells, Q = 32: 2944 -> 3038 us per step) and the small-domain kernels nothing.
 #pragma once
 #include <stdint.h>
 
 namespace qlbm {
 
-// Mantissa of a double as a signed fixed-point number, bit 58 the leading bit
-// of exponent field E (E >= the value's own field, E >= 1).
-__device__ __forceinline__ int64_t i64_fix_(double x, int E)
+// Exponent field of a double (0 for zero and subnormal numbers).
+__device__ __forceinline__ int exp_field_(double x) { return int((uint32_t(__double2hiint(x)) >> 20) & 0x7FFu); }
+
+// Signed mantissa of a double of exponent field e, leading bit 62 (subnormal numbers: that of field 1).
+__device__ __forceinline__ int64_t i64_mantissa_(double x, int e)
 {
     const uint32_t hi = uint32_t(__double2hiint(x)), lo = uint32_t(__double2loint(x));
-    const int e = int((hi >> 20) & 0x7FFu);
     const uint32_t mh = (hi & 0xFFFFFu) | (e ? 0x100000u : 0u);
-    const uint64_t m = (((uint64_t(mh) << 32) | lo) << 11) >> min(E - max(e, 1) + 5, 63);
-    const int64_t s = int64_t(int32_t(hi) >> 31);
-    return (int64_t(m) ^ s) - s;
+    const int64_t m = int64_t(((uint64_t(mh) << 32) | lo) << 10), s = int64_t(int32_t(hi) >> 31);
+    return (m ^ s) - s;
 }
+// The same as fixed point, bit 59 the leading bit of exponent field E >= e, E >= 1.
+__device__ __forceinline__ int64_t i64_fix_(int64_t m, int e, int E) { return m >> min(E - max(e, 1) + 3, 63); }
 
 // double(Q) rounded to nearest (ties away), |Q| < 2^62; the conversion instruction
 // occupies the FP64 pipe for about 100 cycles per warp, this about 30 issue slots.
@@ -54,7 +62,7 @@ __device__ __forceinline__ double i64_to_double_(int64_t Q)
 __device__ __forceinline__ void i64_indicator_(int64_t s, int64_t d, uint64_t &B, unsigned &e)
 {
     uint64_t us = uint64_t(s < 0 ? -s : s), ud = uint64_t(d < 0 ? -d : d);
-    const int sh = __clzll(int64_t(us | ud)) - 1;  // |s|, |d| < 2^61
+    const int sh = __clzll(int64_t(us | ud)) - 1;  // |s|, |d| < 2^62
     us <<= sh;
     ud <<= sh;
     const uint64_t b = __umul64hi(us, us) + __umul64hi(ud, (ud >> 1) + (ud >> 3) - (ud >> 6));
@@ -79,50 +87,63 @@ template <int N>
 __device__ __forceinline__ void weno5_faces_i64(const double (&a)[N], const double (&b)[N], const double (&g)[N],
                                                 const double (&c)[N], const double (&f0)[N], double (&h)[N])
 {
-    const uint32_t kAbs = 0x7FFFFFFFu;
-    int E[N];
-    int64_t xa[N], xb[N], xg[N], xc[N];
+    int E[3][N];         // exponent of each stencil
+    int64_t x[3][2][N];  // its two differences
     uint64_t B[3][N], W[3][N], S[N];
     unsigned e[3][N];
 #pragma unroll
     for (int k = 0; k < N; ++k) {
-        const uint32_t m = max(max(uint32_t(__double2hiint(a[k])) & kAbs, uint32_t(__double2hiint(b[k])) & kAbs),
-                               max(uint32_t(__double2hiint(g[k])) & kAbs, uint32_t(__double2hiint(c[k])) & kAbs));
-        E[k] = max(int(m >> 20), 1);
+        const int ea = exp_field_(a[k]), eb = exp_field_(b[k]), eg = exp_field_(g[k]), ec = exp_field_(c[k]);
+        E[0][k] = max(max(ea, eb), 1);
+        E[1][k] = max(max(eb, eg), 1);
+        E[2][k] = max(max(eg, ec), 1);
+        const int64_t ma = i64_mantissa_(a[k], ea), mb = i64_mantissa_(b[k], eb), mg = i64_mantissa_(g[k], eg),
+                      mc = i64_mantissa_(c[k], ec);
+        x[0][0][k] = i64_fix_(ma, ea, E[0][k]);
+        x[0][1][k] = i64_fix_(mb, eb, E[0][k]);
+        x[1][0][k] = i64_fix_(mb, eb, E[1][k]);
+        x[1][1][k] = i64_fix_(mg, eg, E[1][k]);
+        x[2][0][k] = i64_fix_(mg, eg, E[2][k]);
+        x[2][1][k] = i64_fix_(mc, ec, E[2][k]);
     }
 #pragma unroll
-    for (int k = 0; k < N; ++k) {
-        xa[k] = i64_fix_(a[k], E[k]);
-        xb[k] = i64_fix_(b[k], E[k]);
-        xg[k] = i64_fix_(g[k], E[k]);
-        xc[k] = i64_fix_(c[k], E[k]);
-    }
+    for (int k = 0; k < N; ++k)
+        i64_indicator_(x[0][0][k] + x[0][1][k] + (x[0][1][k] >> 2) + (x[0][1][k] >> 3), x[0][1][k], B[0][k], e[0][k]);
 #pragma unroll
-    for (int k = 0; k < N; ++k) i64_indicator_(xa[k] + xb[k] + (xb[k] >> 2) + (xb[k] >> 3), xb[k], B[0][k], e[0][k]);
+    for (int k = 0; k < N; ++k)
+        i64_indicator_(x[1][1][k] - (x[1][0][k] >> 1) - (x[1][0][k] >> 3), x[1][0][k], B[1][k], e[1][k]);
 #pragma unroll
-    for (int k = 0; k < N; ++k) i64_indicator_(xg[k] - (xb[k] >> 1) - (xb[k] >> 3), xb[k], B[1][k], e[1][k]);
-#pragma unroll
-    for (int k = 0; k < N; ++k) i64_indicator_(xc[k] - xg[k] - (xg[k] >> 2) - (xg[k] >> 3), xg[k], B[2][k], e[2][k]);
-    // products of two indicators, squared, relative to the smallest indicator's
-    // exponent: 1 : 6 : 3 are the ideal weights
-#pragma unroll
-    for (int k = 0; k < N; ++k) {
-        const unsigned em = max(max(e[0][k], e[1][k]), e[2][k]);
-        const uint64_t M23 = __umul64hi(B[1][k], B[2][k]), M13 = __umul64hi(B[0][k], B[2][k]),
-                       M12 = __umul64hi(B[0][k], B[1][k]);
-        W[0][k] = __umul64hi(M23, M23) >> min(2u * (em - e[0][k]) + 5u, 63u);
-        W[1][k] = 6 * (__umul64hi(M13, M13) >> min(2u * (em - e[1][k]) + 5u, 63u));
-        W[2][k] = 3 * (__umul64hi(M12, M12) >> min(2u * (em - e[2][k]) + 5u, 63u));
-        S[k] = W[0][k] + W[1][k] + W[2][k];  // in [2^55, 2^62.4)
-    }
+    for (int k = 0; k < N; ++k)
+        i64_indicator_(x[2][1][k] - x[2][0][k] - (x[2][0][k] >> 2) - (x[2][0][k] >> 3), x[2][0][k], B[2][k], e[2][k]);
+    // products of two indicators, squared, times the ideal weights 1 : 6 : 3; the weight of stencil q is
+    // W[q] 2^(h[q] - s[q]) up to a common factor, h = 2 e - 4 E and s = 5, 2, 3, its differences have exponent E
+    int T[N], n[N];
     int64_t Nm[N], d[N];
     uint64_t x0[N];
 #pragma unroll
     for (int k = 0; k < N; ++k) {
-        const int n = __clz(int(S[k] >> 32)) - 1;
-        S[k] <<= n;
-        Nm[k] = __mul64hi(int64_t(W[0][k] << n), 2 * xa[k] + 5 * xb[k]) +
-                __mul64hi(int64_t(W[1][k] << n), xb[k] + 2 * xg[k]) + __mul64hi(int64_t(W[2][k] << n), 4 * xg[k] - xc[k]);
+        const uint64_t M23 = __umul64hi(B[1][k], B[2][k]), M13 = __umul64hi(B[0][k], B[2][k]),
+                       M12 = __umul64hi(B[0][k], B[1][k]);
+        W[0][k] = __umul64hi(M23, M23);
+        W[1][k] = 3 * (__umul64hi(M13, M13) >> 2);
+        W[2][k] = 3 * (__umul64hi(M12, M12) >> 2);
+    }
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        const int h0 = 2 * int(e[0][k]) - 4 * E[0][k], h1 = 2 * int(e[1][k]) - 4 * E[1][k], h2 = 2 * int(e[2][k]) - 4 * E[2][k];
+        const int hm = max(max(h0, h1), h2);
+        // the weights' sum relative to the smallest indicator's exponent, in [2^55, 2^62.4)
+        S[k] = (W[0][k] >> min(hm - h0 + 5, 63)) + (W[1][k] >> min(hm - h1 + 2, 63)) + (W[2][k] >> min(hm - h2 + 3, 63));
+        // 6 times the weighted sum of the candidates times 2^-T: the largest term's weight shifted by 2 (three terms
+        // below 2^60.8)
+        const int g0 = h0 + E[0][k] - 5, g1 = h1 + E[1][k] - 2, g2 = h2 + E[2][k] - 3;
+        const int gm = max(max(g0, g1), g2) + 2;
+        T[k] = gm - hm;
+        Nm[k] = __mul64hi(int64_t(W[0][k] >> min(gm - g0, 63)), 2 * x[0][0][k] + 5 * x[0][1][k]) +
+                __mul64hi(int64_t(W[1][k] >> min(gm - g1, 63)), x[1][0][k] + 2 * x[1][1][k]) +
+                __mul64hi(int64_t(W[2][k] >> min(gm - g2, 63)), 4 * x[2][0][k] - x[2][1][k]);
+        n[k] = __clz(int(S[k] >> 32)) - 1;
+        S[k] <<= n[k];
     }
     // X = 2^125 / S: x0 from the FP32 reciprocal (relative error about 2^-22),
     // then x0 (1 + d + d^2) with d = 1 - S x0 (Householder's third-order step)
@@ -140,10 +161,11 @@ __device__ __forceinline__ void weno5_faces_i64(const double (&a)[N], const doub
 #pragma unroll
     for (int k = 0; k < N; ++k) {
         const int64_t X = int64_t(x0[k] + uint64_t(__mul64hi(d[k] << 20, int64_t(x0[k] >> 1)) >> 16));
-        // Q = 3 (h - f0) 2^(58 - (E - 1023)): one third of the unit, by its exponent
-        const int64_t Q = __mul64hi(Nm[k] << 2, X);
-        const int unit = E[k] >= 61 ? 0x3FD55555 + ((E[k] - 1081) << 20) : 0;
-        h[k] = fma(i64_to_double_(Q), __hiloint2double(E[k] == 0x7FF ? 0x7FF80000 : unit, 0x55555555), f0[k]);
+        // Q = 6 (h - f0) 2^(1079 - T - n): a sixth of the unit, by its exponent
+        const int64_t Q = __mul64hi(Nm[k], X);
+        const int unit = T[k] + n[k] >= 60 ? 0x3FD55555 + ((T[k] + n[k] - 1080) << 20) : 0;
+        const bool nan = max(max(E[0][k], E[1][k]), E[2][k]) == 0x7FF;
+        h[k] = fma(i64_to_double_(Q), __hiloint2double(nan ? 0x7FF80000 : unit, 0x55555555), f0[k]);
     }
 }
 __device__ __forceinline__ double weno5_face_i64(double a, double b, double g, double c, double f0)

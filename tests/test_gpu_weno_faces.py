@@ -73,3 +73,28 @@ def _power_of_two_rows():
 @pytest.mark.parametrize("repeat", [1, 160])
 def test_weights_of_powers_of_two(gpu, repeat):
     _check_advection(gpu, _power_of_two_rows(), 8, repeat)
+
+
+def _steep_rows():
+    """Positive rows whose neighbouring values differ by large factors: tails that fall and rise by e^5 and e^12 per cell, a flat
+    tail beside a jump of 22 and 25 decades, a Gaussian population across a temperature jump, random factors, and (values of
+    ordinary size) random data and jumps by 1.5, 2, 3 and 8."""
+    rng = np.random.default_rng(17)
+    u = lambda n, amp: 1.0 + amp * rng.uniform(0, 1, n)
+    out = [np.exp(-5.0 * np.arange(12)) * u(12, 0.1), np.exp(-60.0 + 5.0 * np.arange(12)) * u(12, 0.1),
+           np.exp(-12.0 * np.arange(6)) * u(6, 0.1), np.exp(-72.0 + 12.0 * np.arange(7)) * u(7, 0.1)]
+    for tail, high in ((1e-25, 1.0), (1e-25, 1e-3), (1e-22, 1.0)):
+        out += [tail * u(8, 0.3), high * u(8, 0.3)]
+    T = np.concatenate([np.full(6, 0.4), np.linspace(0.4, 1.3, 7), np.full(6, 1.3)])
+    for p in (3.0, 5.0, 7.0):
+        f = np.exp(-p * p / (2 * T)) * u(len(T), 1e-3)
+        out += [f, f[::-1]]
+    out += [np.exp(rng.uniform(-12, 12, 200)), rng.uniform(0, 1, 200)]
+    for r in (1.5, 2.0, 3.0, 8.0):
+        out += [u(5, 0.01), u(7, 0.01) / r]
+    return np.concatenate(out)
+
+
+@pytest.mark.parametrize("repeat", [1, 250])
+def test_steep_rows_keep_the_relative_precision_of_small_values(gpu, repeat):
+    _check_advection(gpu, _steep_rows(), 8, repeat)
