@@ -72,11 +72,15 @@ __device__ __forceinline__ double2 sub2(double2 a, double2 b) { return make_doub
 __device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
 
-// sqrt(x) for normal x > 0.  FP64: from the hardware's reciprocal square root r0
-// (PTX rsqrt.approx.ftz.f64), x r0 (1 + e/2 + 3 e^2/8) with e = 1 - x r0^2.
+// sqrt(x) for x > 0.  FP64: from the hardware's reciprocal square root r0
+// (PTX rsqrt.approx.ftz.f64), x r0 (1 + e/2 + 3 e^2/8) with e = 1 - x r0^2; at most 0.76 units in the last
+// place from the root (x rsqrt(x): 1.50; measured over 4e6 values each in six ranges).  The approximation
+// takes subnormal numbers for zero: they, and what is not a positive finite number, take x rsqrt(x).
 __device__ __forceinline__ float sqrt_(float x) { return x * rsqrtf(x); }
+static __device__ __noinline__ double sqrt_special_(double x) { return x * rsqrt(x); }
 __device__ __forceinline__ double sqrt_(double x)
 {
+    if (unsigned(__double2hiint(x) - 0x00100000) >= 0x7FE00000u) return sqrt_special_(x);
     double r;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
     const double t = x * r, e = fma(-t, r, 1.0);
@@ -152,11 +156,15 @@ __device__ __forceinline__ float rcp_<float>(float x)
 }
 // FP64: the hardware's approximation (PTX rcp.approx.ftz.f64, relative error
 // e < 2^-19.9 measured) and one third-order step r (1 + e + e^2), three FP64
-// instructions instead of the division's five; at most one unit in the last
-// place from the rounded quotient (measured over 10^8 values).
+// instructions instead of the division's five; at most 0.508 units in the last
+// place from 1 / x (measured over 4e6 values each in six ranges; the division 0.5).  Zeros,
+// infinities (a Knudsen number may be infinite: no collisions), NaN, subnormal numbers and those
+// with subnormal reciprocals take the division.
+static __device__ __noinline__ double rcp_special_(double x) { return 1.0 / x; }
 template <>
 __device__ __forceinline__ double rcp_<double>(double x)
 {
+    if (unsigned((__double2hiint(x) & 0x7FFFFFFF) - 0x00100000) >= 0x7FC00000u) return rcp_special_(x);
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
     const double e = fma(-x, r, 1.0);
