@@ -102,23 +102,27 @@ __device__ __forceinline__ Real log_(Real x);
 template <>
 __device__ __forceinline__ float log_<float>(float x) { return logf(x); }
 // FP64: the library's log takes 32 FP64 instructions (2083 cycles per warp
-// measured), this 15: table-driven reduction (P. T. P. Tang, ACM TOMS 16, 1990)
+// measured), this 22: table-driven reduction (P. T. P. Tang, ACM TOMS 16, 1990)
 // x = 2^e m with m in [0.707, 1.414), m = c (1 + r) with c at the middle of one of
 // 128 intervals (c = 1 on the two next to 1), |r| < 2^-7, and the Taylor series of
-// log(1 + r) to r^8.  e log 2 + log c is held in two parts, the leading one exact
-// (multiples of 2^-42), so the result is within 0.6 units in the last place.  For
-// finite normal x > 0; others give NaN.
+// log(1 + r) to r^8.  r is held exactly (the rounded product's difference from 1 and the product's
+// error), e log 2 + log c in two parts, the leading one exact (multiples of 2^-42), and the sum of
+// the leading parts keeps its error.  At most 0.52 units in the last place from log x (4e6 values each in
+// six ranges, one of them next to 1; the library 0.55; with r and the sum rounded, 15
+// instructions, it was 0.995 next to 1).  Subnormal numbers and what is not a positive finite
+// number take the library's.
 #ifdef QL_LOGTAB
+static __device__ __noinline__ double log_special_(double x) { return log(x); }
 template <>
 __device__ __forceinline__ double log_<double>(double x)
 {
     const int hi = __double2hiint(x);
-    if (unsigned(hi - 0x00100000) >= 0x7FE00000u) return __hiloint2double(0x7FF80000, 0);
+    if (unsigned(hi - 0x00100000) >= 0x7FE00000u) return log_special_(x);
     const int d = hi - 0x3FE6A000;
     const int e = d >> 20, j = (d >> 13) & 127;
     const double m = __hiloint2double(hi - (e << 20), __double2loint(x));
     const double2 t = QL_LOGTAB[2 * j];  // 1 / c, leading part of log c
-    const double r = fma(m, t.x, -1.0), r2 = r * r;
+    const double q = m * t.x, rl = fma(m, t.x, -q), r = q - 1.0, r2 = r * r;
     double p = fma(r, -1.0 / 8.0, 1.0 / 7.0);
     p = fma(r, p, -1.0 / 6.0);
     p = fma(r, p, 1.0 / 5.0);
@@ -127,8 +131,9 @@ __device__ __forceinline__ double log_<double>(double x)
     p = fma(r, p, -1.0 / 2.0);
     // double(e), exact: 2^52 + 2^51 + e as bits, less the constant
     const double ed = __hiloint2double(0x43380000 + (e >> 31), e) - 6755399441055744.0;
-    const double lo = fma(r2, p, fma(ed, QL_LOGTAB[257].y, QL_LOGTAB[2 * j + 1].x));
-    return fma(ed, QL_LOGTAB[257].x, t.y) + (r + lo);
+    const double lo = fma(r2, p, fma(ed, QL_LOGTAB[257].y, QL_LOGTAB[2 * j + 1].x)) + fma(-r, rl, rl);
+    const double h = fma(ed, QL_LOGTAB[257].x, t.y), s = h + r;  // h is zero or larger than r
+    return s + (((h - s) + r) + lo);
 }
 #else
 template <>
