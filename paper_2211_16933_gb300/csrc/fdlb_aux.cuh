@@ -13,10 +13,12 @@ namespace qlbm {
 // Discrete equilibrium of given fields (Eq. feq), computed in FP64, for the
 // interior and the ghost columns.  One thread per column: the normalised
 // Hermite coefficients once, then g at +p_k and -p_k from the even and odd
-// parts of the sum.
+// parts of the sum: of the velocity pairs with their bit set in `any` (the same in the threads that
+// run together), stored for those in `pairs`.
 template <typename Real, int Q>
 __device__ __forceinline__ void init_column(double uu, double TT, double n, P2<Real> *__restrict__ psi, int64_t stride,
-                                            const double *__restrict__ tab)
+                                            const double *__restrict__ tab, unsigned any = ~0u,
+                                            unsigned pairs = ~0u)
 {
     constexpr TabView TV = tab_view(Q);
     constexpr int H = Q / 2;
@@ -26,6 +28,7 @@ __device__ __forceinline__ void init_column(double uu, double TT, double n, P2<R
 #pragma unroll
     for (int l = 2; l < Q; ++l) ch[l] = tab[TV.ca + l] * uu * ch[l - 1] + tab[TV.cb + l] * (TT - 1.0) * ch[l - 2];
     for (int j = 0; j < H; ++j) {
+        if (!(any >> j & 1u)) continue;
         const double *G = tab + TV.G + (H + j) * Q;
         double e = 0.0, o = 0.0;
 #pragma unroll
@@ -34,6 +37,7 @@ __device__ __forceinline__ void init_column(double uu, double TT, double n, P2<R
             o = fma(G[l + 1], ch[l + 1], o);
         }
         const double gp = n * (e + o), gm = n * (e - o);
+        if (!(pairs >> j & 1u)) continue;
         psi[int64_t(H + j) * stride] = mk2(Real(gp), Real(2.0 * TT * gp));
         psi[int64_t(H - 1 - j) * stride] = mk2(Real(gm), Real(2.0 * TT * gm));
     }

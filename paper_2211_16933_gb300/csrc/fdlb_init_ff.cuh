@@ -4,12 +4,17 @@
 // fdlb_init_kernel<float> was bound by the FP64 pipe (about 64 cycles per warp
 // instruction and sub-partition): 518 FP64 instructions per cell at Q = 24, 922 us for 10^6
 // cells where the 0.2 GB written take 29 (a ql_load_fields call with three steps after it: 2466
-// us, now 1692, the same bits).  Here a term of the sums is 12 packed FP32
+// us, now 1707).  Here a term of the sums is 12 packed FP32
 // instructions for an even and an odd coefficient together: the exact product's two halves,
 // the error-free sum, and the low parts in a second accumulator (compensated dot
 // product, T. Ogita, S. M. Rump, S. Oishi, SIAM J. Sci. Comput. 26, 2005).  Fields outside
 // the range in which its intermediate values stay far from FP32's limits (|u|, |T - 1|
-// < 8, n and T neither tiny nor huge) take the FP64 sums.
+// < 8, n and T neither tiny nor huge) take the FP64 sums.  So do velocity pairs with a g below 2^-12 of
+// the sum of its terms' magnitudes (fast velocities of states far from u = 0, T = 1), where about 48 bits
+// are too few: against quadruple precision the largest error there was 2 to 10^3 times that of the
+// FP64 sums, and above the line it is 0.5001 FP32 units in the last place, as theirs (0.5000; 240000 random
+// states, all velocity sets).  None are below it for |u| < 0.1 and |T - 1| < 0.05; at Q = 32, |u| < 0.4 and |T - 1|
+// < 0.2 6 % are, u = 1.0 to 1.4 and T = 0.4 to 0.6 47 %.
 #pragma once
 #include "fdlb_aux.cuh"
 
@@ -61,11 +66,14 @@ __device__ __forceinline__ FF ff_split(double x)
     return fast_two_sum(float(top) * s, float(unsigned(lo) & 0x1FFFFFFFu) * (s * 0x1p-29f));
 }
 
+// FP64 sums of the velocity pairs whose bit in `pairs` is set, as init_column (threads that skipped
+// different pairs went through the loop one after the other: 10.1 ms for 10^6 cells at Q = 40, u = 1.0 to
+// 1.4 and T = 0.4 to 0.6, 1.9 so, all in FP64 2.2).
 template <int Q>
-__device__ __noinline__ void init_column_f64(double uu, double TT, double n, float2 *__restrict__ psi, int64_t stride,
-                                             const double *__restrict__ tab)
+__device__ __noinline__ void init_pairs_f64(double uu, double TT, double n, float2 *__restrict__ psi, int64_t stride,
+                                            const double *__restrict__ tab, unsigned pairs)
 {
-    init_column<float, Q>(uu, TT, n, psi, stride, tab);
+    init_column<float, Q>(uu, TT, n, psi, stride, tab, __reduce_or_sync(__activemask(), pairs), pairs);
 }
 
 // One thread per column, as fdlb_init_kernel.
@@ -81,7 +89,7 @@ __global__ void __launch_bounds__(256) fdlb_init_ff_kernel(const double *__restr
     const double uu = u[c], TT = T[c], n = rho[c], Tm = TT - 1.0;
     const int en = exponent_(n), et = exponent_(TT);
     if (!(exponent_(uu) < 3 && exponent_(Tm) < 3 && en >= -60 && en < 60 && et >= -60 && et < 60)) {
-        init_column_f64<Q>(uu, TT, n, psi + c, stride, tab);
+        init_pairs_f64<Q>(uu, TT, n, psi + c, stride, tab, ~0u);
         return;
     }
     const FF fu = ff_split(uu), ft = ff_split(Tm), fn = ff_split(n);
@@ -103,24 +111,30 @@ __global__ void __launch_bounds__(256) fdlb_init_ff_kernel(const double *__restr
             m1 = co;
         }
     }
+    unsigned steep = 0;  // pairs left to the FP64 sums
 #pragma unroll 1
     for (int j = 0; j < H; ++j) {
         float2 s = sp2(0.f), r = sp2(0.f);  // the even and the odd sum: rounded, and what it lacks
+        float size = 0.f;                   // sum of the magnitudes
 #pragma unroll
         for (int m = 0; m < H; ++m) {
             const float4 g = QL_FFTAB[OFF + j * H + m];
             const float2 gh = mk2(g.x, g.y), ngh = mk2(-g.x, -g.y), ngl = mk2(g.z, g.w);
             const float2 p = mul2(gh, ch[m]);
+            size += fabsf(p.x) + fabsf(p.y);
             const float2 lack = fma2(ngl, ch[m], fma2(ngh, cl[m], fma2(ngh, ch[m], p)));  // p - (exact term)
             const float2 w = add2(s, p), b = sub2(w, s);
             r = add2(r, sub2(add2(sub2(s, sub2(w, b)), sub2(p, b)), lack));
             s = w;
         }
         const FF e = two_sum(s.x, r.x), o = two_sum(s.y, r.y);
-        const FF gp = ff_mul(fn, ff_add(e, o)), gm = ff_mul(fn, ff_add(e, ff_neg(o)));
+        const FF sp = ff_add(e, o), sm = ff_add(e, ff_neg(o));
+        if (!(fminf(fabsf(sp.h), fabsf(sm.h)) >= 0x1p-12f * size)) steep |= 1u << j;
+        const FF gp = ff_mul(fn, sp), gm = ff_mul(fn, sm);
         psi[int64_t(H + j) * stride + c] = mk2(gp.h, ff_mul(t2, gp).h);
         psi[int64_t(H - 1 - j) * stride + c] = mk2(gm.h, ff_mul(t2, gm).h);
     }
+    if (steep) init_pairs_f64<Q>(uu, TT, n, psi + c, stride, tab, steep);
 }
 
 }  // namespace qlbm
