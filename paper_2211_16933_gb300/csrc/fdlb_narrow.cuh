@@ -39,6 +39,7 @@ __global__ void __launch_bounds__(kThreads, 2) fdlb_narrow_kernel(NarrowArgs s)
     __shared__ Real s_part[6][NG][SEG];
     __shared__ Real s_n[SEG], s_u[SEG], s_T[SEG], s_q[SEG], s_lnn[SEG], s_lnT[SEG];
     __shared__ Real s_chi[RET ? SEG : 1], s_lnchi[RET ? SEG : 1], s_dn[RET ? H : 1][RET ? 32 : 1];
+    __shared__ Real s_bn[RET ? SEG + 2 * kNarrowBall : 1], s_bk[RET ? 2 * kNarrowBall + 1 : 1];
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const StageArgs &a = s.a;
@@ -71,16 +72,26 @@ __global__ void __launch_bounds__(kThreads, 2) fdlb_narrow_kernel(NarrowArgs s)
             }
         }
     }
-    if (RET && t >= kThreads - 64 && t - (kThreads - 64) < SEG) {
-        // nbar as fdlb_fm_kernel forms it, then Eq. (chi_ret), while the loads above are in flight
-        const int c = t - (kThreads - 64);
+    if (RET && t >= kThreads - 64) {
+        // nbar as fdlb_fm_kernel forms it, then Eq. (chi_ret), by two warps while the loads above are in
+        // flight.  The ball's weights (one FP64 conversion each) and densities go through shared memory: with
+        // each thread fetching and converting all of its own, balls of 8 and 16 cells were slower than on
+        // tiles with the average as a launch of its own (us per step; tiles, each its own, this: Q = 8, 16384 cells, 16 cells:
+        // 24.6, 52.7, 24.5; Q = 20, 5000 cells, 8 cells: 35.0, 30.8, 18.4).
+        const int c = t - (kThreads - 64), W = s.f.W;
         const Real *n = static_cast<const Real *>(s.f.n);
-        Real nbar = 0.f;
-        for (int d = 0; d <= 2 * s.f.W; ++d)
-            nbar = fma_(Real(s.f.K[d]), fm_density<Real>(s.f, n, i0 - kHalo + c - s.f.W + d), nbar);
-        const Real chi = chi_of_nbar_(a, nbar);
-        s_chi[c] = chi;
-        s_lnchi[c] = log_(chi);
+        const double weight = s.f.K[min(c, 2 * W)];  // in flight beside the densities
+        for (int e = c; e < SEG + 2 * W; e += 64) s_bn[e] = fm_density<Real>(s.f, n, i0 - kHalo - W + e);
+        if (c <= 2 * W) s_bk[c] = Real(weight);
+        asm volatile("bar.sync 1, 64;" ::: "memory");
+        if (c < SEG) {
+            Real nbar = 0.f;
+#pragma unroll 4
+            for (int d = 0; d <= 2 * W; ++d) nbar = fma_(s_bk[d], s_bn[c + d], nbar);
+            const Real chi = chi_of_nbar_(a, nbar);
+            s_chi[c] = chi;
+            s_lnchi[c] = log_(chi);
+        }
     }
 #pragma unroll
     for (int k = 0; k < LOADS; ++k) {
