@@ -190,7 +190,11 @@ typedef struct {
  * Errors: QL_EINVAL (bad sizes, dt <= 0, eta0 out of range, init kind needs
  * another bc, bad chi_mode), QL_EUNSUPPORTED (Q; a chi_RET-FM ball reaching
  * more than QL_FM_MAX_HALFWIDTH cells), QL_ENOMEM, QL_ECUDA.  On error *out is
- * NULL. */
+ * NULL.
+ * FP64 domains of up to 131072 cells take 5 + Q / 2 (phi, theta) pairs per cell besides the three
+ * states, and FP32 domains of up to 16384 cells with chi_RET-FM a second density array: if
+ * these cannot be allocated the solver is created without (same results, slower kernels; sets
+ * other than Q = 8, 16, 20, 24, 32, 40 need them, for at least 32 cells at a time). */
 ql_status ql_create(const ql_velset *vs, const ql_grid *grid, double denseness, double kn,
                     const ql_bc *bc, const ql_init *init, const ql_opts *opts, ql_ctx **out);
 

@@ -348,6 +348,33 @@ static void destroy_buffers(ql_ctx *c)
     dev_free(c, c->d_ch);
 }
 
+// The buffers that only the small-domain kernels need, allocated after everything else: where
+// they do not fit, velocity sets with tiles run the tile kernels (which give the same bits), and the
+// others take smaller chunks.  False: not even one chunk of 32 cells.
+static bool small_domain_buffers(ql_ctx *c)
+{
+    if (c->narrow && c->chi_mode == QL_CHI_RET_FM) {
+        c->d_n2 = dev_alloc(c, 4 * size_t(c->nx));
+        if (!c->d_n2) {
+            c->narrow = false;
+            (void)cudaGetLastError();
+        }
+    }
+    if (c->cells) c->ccols = std::min<int64_t>((c->nx + 31) / 32 * 32, kCellChunk);
+    while (c->cells) {
+        c->d_coef = dev_alloc(c, 5 * size_t(c->ccols) * c->elem);
+        c->d_ch = c->d_coef ? dev_alloc(c, size_t(c->Q / 2) * size_t(c->ccols) * c->elem) : nullptr;
+        if (c->d_ch) break;
+        (void)cudaGetLastError();
+        dev_free(c, c->d_coef);
+        c->d_coef = nullptr;
+        if (!c->lq) c->cells = false;
+        else if (c->ccols == 32) return false;
+        c->ccols = std::max<int64_t>(32, c->ccols / 2 / 32 * 32);
+    }
+    return true;
+}
+
 extern "C" {
 
 ql_status ql_create(const ql_velset *vs, const ql_grid *grid, double denseness, double kn, const ql_bc *bc,
@@ -479,12 +506,6 @@ ql_status ql_create(const ql_velset *vs, const ql_grid *grid, double denseness, 
     c->cells = c->lq || (!c->fault && c->precision == QL_FP64 && c->nx <= kCellChunk);
     c->narrow = !c->lq && !c->fault && c->precision == QL_FP32 && c->nx <= kNarrowCells &&
                 (c->chi_mode == QL_CHI_SET || c->fm_w <= kNarrowBall);
-    if (c->cells) {
-        c->ccols = std::min<int64_t>((c->nx + 31) / 32 * 32, kCellChunk);
-        c->d_coef = dev_alloc(c, 5 * size_t(c->ccols) * c->elem);
-        c->d_ch = dev_alloc(c, size_t(c->Q / 2) * size_t(c->ccols) * c->elem);
-        if (!c->d_coef || !c->d_ch) return bail(QL_ENOMEM, "per-cell buffer allocation failed");
-    }
     if (c->lq) {
         c->d_lqtab = static_cast<double *>(dev_alloc(c, sizeof(double) * lqtab.size()));
         if (!c->d_lqtab) return bail(QL_ENOMEM, "large-Q table allocation failed");
@@ -497,8 +518,7 @@ ql_status ql_create(const ql_velset *vs, const ql_grid *grid, double denseness, 
         c->d_fmk = static_cast<double *>(dev_alloc(c, sizeof(double) * (2 * c->fm_w + 1)));
         c->d_n = dev_alloc(c, real * c->nx);
         c->d_nbar = dev_alloc(c, real * c->stride);
-        if (c->narrow) c->d_n2 = dev_alloc(c, real * c->nx);
-        if (!c->d_fmk || !c->d_n || !c->d_nbar || (c->narrow && !c->d_n2)) return bail(QL_ENOMEM, "chi_RET-FM buffer allocation failed");
+        if (!c->d_fmk || !c->d_n || !c->d_nbar) return bail(QL_ENOMEM, "chi_RET-FM buffer allocation failed");
         std::vector<double> K(2 * c->fm_w + 1);
         fm_weights(c->dx, c->sigma, c->fm_w, K.data());
         e = cudaMemcpyAsync(c->d_fmk, K.data(), sizeof(double) * K.size(), cudaMemcpyHostToDevice, c->stream);
@@ -506,6 +526,7 @@ ql_status ql_create(const ql_velset *vs, const ql_grid *grid, double denseness, 
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);  // K goes out of scope
         if (e != cudaSuccess) return bail(QL_ECUDA, std::string("chi_RET-FM set-up: ") + cudaGetErrorString(e));
     }
+    if (!small_domain_buffers(c)) return bail(QL_ENOMEM, "per-cell buffer allocation failed");
     e = cudaMemcpyAsync(c->d_tab64, g_tab, sizeof(double) * kTabTotal, cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_err, 0, 256, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->buf[0], 0, state_bytes, c->stream);
