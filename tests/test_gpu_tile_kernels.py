@@ -1,10 +1,10 @@
 """The tile stage kernels of the solver, at the smallest domains that take them (a few cells more than the small-domain
 kernels do: 131072 in FP64, 16384 in FP32), for every compiled velocity set, both chi modes and both precisions.
 
-A periodic domain of three equal periods must give, period by period, the bits of one period alone, which is small
-enough for the small-domain kernels (same arithmetic in the same order).  Lengths, Knudsen numbers and the denseness are
-chosen so that cell size, ball and relaxation time are the same numbers in both: products of small integers and
-powers of two.  Fixed boundaries are compared with the oracle's right-hand side, to 1e-11 (FP64) and 2e-5 (FP32) of its
+A periodic domain of four equal periods must give, period by period, the bits of one period alone, which is small
+enough for the small-domain kernels (same arithmetic in the same order).  Lengths and Knudsen numbers differ by factors
+of four, so that cell size, ball and relaxation time are the same numbers in both, whatever the order in which they are
+rounded.  Fixed boundaries are compared with the oracle's right-hand side, to 1e-11 (FP64) and 2e-5 (FP32) of its
 largest value, the tolerances of the other right-hand-side tests."""
 import numpy as np
 import pytest
@@ -13,16 +13,15 @@ import oracle as O
 from paper_2211_16933_gb300 import inputs
 
 pytestmark = pytest.mark.gpu
-PERIOD = {0: 43691, 1: 5462}  # three of them: 131073 and 16386 cells, with ragged last tiles
+PERIOD = {0: 32769, 1: 4097}  # four of them: 131076 and 16388 cells, with ragged last tiles
 
 
 def _solver(q, precision, Q, nx, periods, ball):
     """`periods` periods of nx cells each; ball: cells that the chi_RET-FM ball reaches on each side (None: chi_SET)."""
     length, El = nx * 2.0 ** -16, 0.25
-    # one period has kn = 3 m, three have m; sigma = El kn length = (ball - 1/4) dx for m to 24 bits
-    m = 2.0 ** -8 if ball is None else float(np.float32((4 * ball - 1) * 2.0 ** -16 / (3 * length)))
+    kn = 2.0 ** -6 if ball is None else (ball - 0.25) * 2.0 ** -16 / (El * length)  # sigma = El kn length
     rho, u, T = inputs.smooth_periodic_fields(nx, seed=Q)
-    s = q.Solver(Q, periods * nx, periods * length, 2e-7, El, 3.0 * m / periods, bc=q.QL_BC_PERIODIC,
+    s = q.Solver(Q, periods * nx, periods * length, 2e-7, El, kn / periods, bc=q.QL_BC_PERIODIC,
                  init_kind=q.QL_INIT_FIELDS, rho=np.tile(rho, periods), u=np.tile(u, periods), T=np.tile(T, periods),
                  precision=precision, chi_mode=q.QL_CHI_SET if ball is None else q.QL_CHI_RET_FM)
     ph, th = s.state()
@@ -36,24 +35,24 @@ def _solver(q, precision, Q, nx, periods, ball):
 @pytest.mark.parametrize("Q", [8, 16, 20, 24, 32, 40])
 def test_tile_kernels_give_the_bits_of_the_small_domain_kernels(gpu, Q, ball, precision):
     nx = PERIOD[precision]
-    one, three = (_solver(gpu, precision, Q, nx, n, ball) for n in (1, 3))
-    assert one.sigma == three.sigma and one.dx == three.dx
-    for a, b in zip(one.rhs(), three.rhs()):
-        np.testing.assert_array_equal(b, np.tile(a, (3, 1)))
-    for s in (one, three):
+    one, four = (_solver(gpu, precision, Q, nx, n, ball) for n in (1, 4))
+    assert one.sigma == four.sigma and one.dx == four.dx
+    for a, b in zip(one.rhs(), four.rhs()):
+        np.testing.assert_array_equal(b, np.tile(a, (4, 1)))
+    for s in (one, four):
         s.step(1)
         s.step(2)
-    for a, b in zip(one.state(), three.state()):
-        np.testing.assert_array_equal(b, np.tile(a, (3, 1)))
+    for a, b in zip(one.state(), four.state()):
+        np.testing.assert_array_equal(b, np.tile(a, (4, 1)))
     one.close()
-    three.close()
+    four.close()
 
 
 @pytest.mark.parametrize("precision", [0, 1])
 @pytest.mark.parametrize("Q", [20, 40])
 @pytest.mark.parametrize("ball", [None, 3])
 def test_tile_kernels_at_fixed_boundaries_match_oracle(gpu, Q, ball, precision):
-    q, nx, El, length = gpu, 3 * PERIOD[precision], 0.3, 1.0
+    q, nx, El, length = gpu, 4 * PERIOD[precision], 0.3, 1.0
     rho, u, T = inputs.smooth_periodic_fields(nx, seed=3)
     ghost = np.array([[rho[0], u[0], T[0]]] * 3 + [[rho[-1], u[-1], T[-1]]] * 3) * [1.01, 1.0, 0.99]
     kn = 0.05 if ball is None else (ball - 0.3) / (El * nx)
