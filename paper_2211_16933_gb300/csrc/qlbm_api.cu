@@ -86,8 +86,11 @@ struct ql_ctx {
 // Q = 16: 785 and 794).
 constexpr int64_t kCellChunk = 131072;
 // FP32 domains of up to this many cells run fdlb_narrow_kernel: it is ahead up to
-// 24576 cells at Q = 32 and 40 and about 16384 at Q = 8 and 16 (fdlb_narrow.cuh).
-constexpr int64_t kNarrowCells = 16384;
+// 24576 cells at Q = 32 and 40 and about 16384 at Q = 16 (fdlb_narrow.cuh).  At Q = 8 with chi_SET it is ahead
+// while its 30-cell CTAs are one wave of three per SM, 13680 cells on 152 SMs (us per step, tiles and
+// this: 13600 cells 14.4, 12.3; 13700 cells 14.4, 14.4; 14400 cells 14.4, 16.4; 16384 cells 15.0, 16.4); with chi_RET-FM the
+// tiles need the ball average's launches and are behind up to 16384 cells (24.6 and 22.5 there).
+constexpr int64_t kNarrowCells = 16384, kNarrowCellsQ8 = 13680;
 
 static std::string g_create_error;
 static std::mutex g_mutex;
@@ -504,8 +507,9 @@ ql_status ql_create(const ql_velset *vs, const ql_grid *grid, double denseness, 
         if (e != cudaSuccess) return bail(QL_ECUDA, std::string("run counters: ") + cudaGetErrorString(e));
     }
     c->cells = c->lq || (!c->fault && c->precision == QL_FP64 && c->nx <= kCellChunk);
-    c->narrow = !c->lq && !c->fault && c->precision == QL_FP32 && c->nx <= kNarrowCells &&
-                (c->chi_mode == QL_CHI_SET || c->fm_w <= kNarrowBall);
+    c->narrow = !c->lq && !c->fault && c->precision == QL_FP32 &&
+                (c->chi_mode == QL_CHI_SET ? c->nx <= (c->Q == 8 ? kNarrowCellsQ8 : kNarrowCells)
+                                           : c->nx <= kNarrowCells && c->fm_w <= kNarrowBall);
     if (c->lq) {
         c->d_lqtab = static_cast<double *>(dev_alloc(c, sizeof(double) * lqtab.size()));
         if (!c->d_lqtab) return bail(QL_ENOMEM, "large-Q table allocation failed");
