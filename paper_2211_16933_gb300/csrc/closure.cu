@@ -1903,13 +1903,15 @@ static ql_status pack(ql_closure *c, const float *x, int B)
 
 static ql_status adam_step(ql_closure *c, float lr);
 
-// The device flags (synchronises): bit 0, a mini-batch index outside the data
-// set; bit 1, a convolution that gave up waiting for its tensor-core products.
+// The device flags (synchronises) raised since the last look at them, and cleared here: bit 0, a
+// mini-batch index outside the data set; bit 1, a kernel that gave up waiting for its
+// tensor-core products (ql_closure_forward does not look: the next call that does reports it).
 static ql_status check_flags(ql_closure *c)
 {
     unsigned bad = 0;
     QC_CUDA(c, cudaMemcpyAsync(&bad, c->bad, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
     QC_CUDA(c, cudaStreamSynchronize(c->stream));
+    if (bad) QC_CUDA(c, cudaMemsetAsync(c->bad, 0, sizeof(unsigned), c->stream));
     if (bad & 2u) return cfail(c, QL_ECUDA, "a convolution gave up waiting for its tensor-core products");
     if (bad & 1u) return cfail(c, QL_EINVAL, "perm holds a sample index outside [0, n); sample 0 was used in its place");
     return QL_OK;
@@ -2150,6 +2152,7 @@ ql_status ql_closure_create(const ql_closure_desc *d, const ql_opts *opts, ql_cl
     cudaError_t e = cudaMemcpyAsync(c->param, h.data(), sizeof(float) * off, cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->m, 0, sizeof(float) * off, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->v, 0, sizeof(float) * off, c->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->bad, 0, sizeof(unsigned), c->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(c->norm, nrm, sizeof(nrm), cudaMemcpyHostToDevice, c->stream);
     for (int l = 0; l < d->layers && e == cudaSuccess; ++l) {
         e = cudaMemsetAsync(c->act[l], 0, sizeof(bf16) * npos * c->layers[l].cin, c->stream);
@@ -2222,7 +2225,6 @@ ql_status ql_closure_train_steps(ql_closure *c, const float *x, const float *y, 
     if (!c || !x || !y || !periodic || !perm || n < 1 || nsteps < 0 || B < 1 || B > c->d.max_batch ||
         (nsteps > 0 && !lr))
         return cfail(c, QL_EINVAL, "bad arguments");
-    QC_CUDA(c, cudaMemsetAsync(c->bad, 0, sizeof(unsigned), c->stream));
     if (nsteps > 0) {
         if (!c->d_step) {
             c->d_step = static_cast<int *>(calloc_dev(c, sizeof(int)));
