@@ -1946,6 +1946,12 @@ static NetArgs net_args(ql_closure *c)
     return a;
 }
 
+static bool overlap(const void *a, size_t na, const void *b, size_t nb)
+{
+    const uintptr_t p = reinterpret_cast<uintptr_t>(a), q = reinterpret_cast<uintptr_t>(b);
+    return p < q + nb && q < p + na;
+}
+
 // Mini-batch of a training run: samples perm[*step B ..] of n (perm null: samples 0 .. B - 1).
 struct BatchIndex {
     const int32_t *perm = nullptr;
@@ -2168,7 +2174,15 @@ ql_status ql_closure_create(const ql_closure_desc *d, const ql_opts *opts, ql_cl
 ql_status ql_closure_forward(ql_closure *c, const float *x, const int32_t *periodic, int64_t B, float *y)
 {
     if (!c || !x || !periodic || !y || B < 1 || B > c->d.max_batch) return cfail(c, QL_EINVAL, "bad arguments");
-    if (chain_supported(int(c->layers.size()), c->d.positions)) {
+    // The whole-network kernel reads a sample while other blocks may already write theirs, so y apart from
+    // periodic, and apart from x or in its place sample by sample; else the kernels per layer, which
+    // pack all of x first and write y last.
+    const size_t cells = size_t(B) * size_t(c->d.positions) * sizeof(float);
+    const size_t ny = cells * size_t(c->d.out_channels);
+    const bool in_place = x == y && c->d.in_channels == c->d.out_channels;
+    if (chain_supported(int(c->layers.size()), c->d.positions) &&
+        (in_place || !overlap(x, cells * size_t(c->d.in_channels), y, ny)) &&
+        !overlap(periodic, size_t(B) * sizeof(int32_t), y, ny)) {
         NetArgs a = net_args(c);
         a.x = x;
         a.per = periodic;
