@@ -52,15 +52,16 @@ def _tensor_roofline(achieved_tflops):
             "kernel": "closure training step: net_kernel, wgrad_kernel, reduce_partials_kernel, loss_step_kernel"}
 
 
-# Sources the stage kernels of each precision are compiled from (the unit and what it includes).
+# Sources the stage kernels of each precision are compiled from (the unit and what the kernels' header includes).
 _STAGE_SOURCES = {
     "fp32": ("paper_2211_16933_gb300/csrc/fdlb_f32.cu", "paper_2211_16933_gb300/csrc/fdlb_impl.cuh",
-             "paper_2211_16933_gb300/csrc/fdlb_kernels.cuh", "paper_2211_16933_gb300/csrc/qlbm_internal.h",
-             "include/qlbm.h"),
-    # the generic large-Q kernels (fdlb_lq.cuh) share the FP64 translation unit but not the tiled kernel's code
+             "paper_2211_16933_gb300/csrc/fdlb_kernels.cuh", "paper_2211_16933_gb300/csrc/weno_i64.cuh",
+             "paper_2211_16933_gb300/csrc/qlbm_internal.h", "include/qlbm.h"),
+    # the small-domain and table-driven kernels (fdlb_cells.cuh, fdlb_lq.cuh) share the FP64 translation unit but not
+    # the tiled kernel's own code
     "fp64": ("paper_2211_16933_gb300/csrc/fdlb_f64.cu", "paper_2211_16933_gb300/csrc/fdlb_impl.cuh",
-             "paper_2211_16933_gb300/csrc/fdlb_kernels.cuh", "paper_2211_16933_gb300/csrc/qlbm_internal.h",
-             "include/qlbm.h"),
+             "paper_2211_16933_gb300/csrc/fdlb_kernels.cuh", "paper_2211_16933_gb300/csrc/weno_i64.cuh",
+             "paper_2211_16933_gb300/csrc/qlbm_internal.h", "include/qlbm.h"),
 }
 
 
@@ -681,8 +682,8 @@ def run_learned(args):
             "config": {"workload": "learned_closure_conv1d_5x64_k5", "pairs": args.pairs, "snapshots": 8,
                        "fine_cells": L.NF, "coarse_cells": L.NC, "fine_steps": S, "epochs": args.epochs,
                        "batch": args.train_batch, "lr": args.lr, "lr_schedule": "cosine to lr/20"},
-            # per training step (graph nodes): gather + pack, 5 convs, mse, 5 wgrads + 5 partial sums,
-            # 4 edge terms + 4 transposed convs, loss sum, adam (with the weight casts), step counter
+            # per training step (graph nodes): the whole network forward and back, the weight gradients, their sums
+            # with Adam and the weight casts, the loss with the step counter
             "gpu_launches": 4 * (nsamp // args.train_batch), "train_conv_tflops": train_tflops,
             "roofline": _tensor_roofline(train_tflops), "data_generation_s": t_gen,
             "train_s": t_train, "loss_per_epoch": losses, "held_out": held,
