@@ -79,12 +79,6 @@ struct ql_ctx {
     std::string err;
 };
 
-// FP64 domains of up to this many cells run their stages as two launches
-// (fdlb_cells.cuh) on velocity sets with tiles too; the per-cell buffers hold as
-// many cells, and other velocity sets run larger domains in chunks of them.  At
-// 131072 cells both forms take the same time (Q = 8: 438 and 447 us per step,
-// Q = 16: 785 and 794).
-constexpr int64_t kCellChunk = 131072;
 // FP32 domains of up to this many cells run fdlb_narrow_kernel: it is ahead up to
 // 24576 cells at Q = 32 and 40 and about 16384 at Q = 16 (fdlb_narrow.cuh).  At Q = 8 with chi_SET it is ahead
 // while its 30-cell CTAs are one wave of three per SM, 13680 cells on 152 SMs (us per step, tiles and

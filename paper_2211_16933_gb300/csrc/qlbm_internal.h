@@ -243,6 +243,11 @@ inline int64_t moment_blocks(int64_t nx) { return (nx + kMomThreads - 1) / kMomT
 // set by the launcher).  K, ghost: the ball's 2 W + 1 weights and
 // the fixed ghost densities, as in FmArgs.
 constexpr int kCellBall = 5;
+// FP64 domains of up to this many cells run their stages so on velocity sets with tiles too; the per-cell
+// buffers hold as many cells, and other velocity sets run larger domains in chunks of them.  At
+// 131072 cells both forms take the same time (Q = 8: 438 and 447 us per step,
+// Q = 16: 785 and 794).
+constexpr int64_t kCellChunk = 131072;
 struct CellArgs {
     StageArgs a;
     const double *tab;

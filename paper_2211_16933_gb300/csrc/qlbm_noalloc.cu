@@ -26,7 +26,8 @@ void set_global_error(const std::string &msg);  // ql_last_error(NULL), qlbm_api
 namespace {
 
 // Scratch for every call: a 256-byte header holding the device error word,
-// then psi^(1) and psi^(2), each Q rows of row_stride (phi, theta) pairs.  Every
+// then psi^(1) and psi^(2), each Q rows of row_stride (phi, theta) pairs, and behind them,
+// where there is room, the per-cell buffers of the small FP64 domains' stages.  Every
 // GPU that loads the library holds this array until the process exits.
 constexpr size_t kScratchBytes = size_t(QL_NOALLOC_SCRATCH_BYTES);
 constexpr size_t kHeaderBytes = 256;
@@ -150,12 +151,27 @@ ql_status ql_step_noalloc(const ql_velset *vs, const ql_grid *grid, double dense
     a.nbar = nullptr;
     a.nout = nullptr;
     a.base = rows;
+    // Small FP64 domains whose per-cell quantities fit behind the stage buffers run the two-launch
+    // stages, as in ql_step (us per step at Q = 32, tiles and these: 1000 cells 197, 67;
+    // 4000 cells 270, 111; 16000 cells 574, 217; 49000 cells 649, 568)
+    const int64_t ccols = (nx + 31) / 32 * 32;
+    const bool cells = opts->precision == QL_FP64 && nx <= kCellChunk &&
+                       kHeaderBytes + 2 * buf + size_t(5 + vs->Q / 2) * size_t(ccols) * elem <= kScratchBytes;
+    CellArgs k = {};
+    k.coef = C + buf;
+    k.ch = C + buf + 5 * size_t(ccols) * elem;
+    k.cs = ccols;
+    k.Q = vs->Q;
     for (int64_t n = 0; n < nsteps && e == cudaSuccess; ++n) {
         void *ins[3] = {rows, B, C}, *outs[3] = {B, C, rows};
         for (int stg = 1; stg <= 3 && e == cudaSuccess; ++stg) {
             a.in = ins[stg - 1];
             a.out = outs[stg - 1];
-            e = opts->precision == QL_FP32 ? launch_stage_f32(vs->Q, stg, a, s) : launch_stage_f64(vs->Q, stg, a, s);
+            k.a = a;
+            k.stage = stg;
+            e = cells                          ? launch_cell_stage(k, false, s)
+                : opts->precision == QL_FP32 ? launch_stage_f32(vs->Q, stg, a, s)
+                                              : launch_stage_f64(vs->Q, stg, a, s);
         }
     }
     unsigned h = 0;
