@@ -40,7 +40,7 @@ def _peaks():
 
 
 def _tensor_roofline(achieved_tflops):
-    """The closure's training step (BF16 mma.sync with FP32 accumulation; convolution FLOPs of the forward and
+    """The closure's training step (BF16 tcgen05.mma with FP32 accumulation; convolution FLOPs of the forward and
     both backward passes) against the measured dense BF16 rate; sustained figure, the step runs for seconds."""
     peaks = _peaks()
     if peaks and "bf16_tflops_sustained" in peaks:

@@ -1257,7 +1257,7 @@ __device__ __forceinline__ void chain_products(uint32_t taddr, uint32_t win, uin
     }
 }
 
-// 32 channels of a position as bf16, into rows c0 / 8 .. of the staged window and of a chunk-major tensor.
+// N channels of a position as bf16 rows of 8 (for the staged window and the chunk-major tensors).
 template <int N>
 __device__ __forceinline__ void pack_row(const float (&v)[N], uint4 (&pk)[N / 8])
 {

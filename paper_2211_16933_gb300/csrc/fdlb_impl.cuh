@@ -66,7 +66,8 @@ cudaError_t QL_FN(upload_tables_)(const double *all)
 
 // One CTA per tile; in FP64, a domain of fewer tiles than the GPU has SMs splits
 // each tile's velocity pairs over up to Q/2 CTAs (FP64 arithmetic, not memory,
-// bounds those small domains).  The split with the least FP64 instructions per
+// bounds those small domains, which come here only when the buffers of the two-launch
+// stages could not be allocated, or with ql_opts.fault).  The split with the least FP64 instructions per
 // thread on the busiest SM is taken: about 8 Q + 170 for the per-cell part, which
 // every CTA of a tile repeats, and Q + 52 per velocity pair.  With chi_RET-FM the densities of the
 // output then come from a separate pass, in the order the stage sums them.
