@@ -16,6 +16,7 @@ from __future__ import annotations
 import argparse
 import hashlib
 import json
+import math
 import os
 import re
 import statistics
@@ -281,9 +282,10 @@ HBM_NOMINAL_GBS = 7900.0  # GB300 HBM3e datasheet bandwidth (context beside the 
 def _hbm_roofline(elem, nx, Q, step_s, precision_name, steps_per_launch, kernel):
     """The stepping kernel against the measured copy bandwidth: 16 words of phi and theta per update per step
     (stage 1 reads 2 / writes 2, stages 2-3 read 4 / write 2).  fdlb_run_kernel: one launch runs
-    steps_per_launch steps; fdlb_stage_kernel: one launch is one stage, a third of a step."""
+    steps_per_launch steps; fdlb_stage_kernel: one launch is one stage, a third of a step (steps_per_launch is the
+    steps that one launch advances in both cases)."""
     bytes_per_step = 16 * elem * nx * Q
-    launches_per_step = 1.0 / steps_per_launch if kernel == "fdlb_run_kernel" else 3.0
+    launches_per_step = 1.0 / steps_per_launch
     achieved = bytes_per_step / step_s / 1e9
     peaks = _peaks()
     if peaks and "hbm_gbs" in peaks:
@@ -302,12 +304,29 @@ def _hbm_roofline(elem, nx, Q, step_s, precision_name, steps_per_launch, kernel)
             "peak_nominal": HBM_NOMINAL_GBS, "frac_of_nominal": achieved / HBM_NOMINAL_GBS}
 
 
+# Domains that the small-domain kernels take (csrc: kCellChunk, kNarrowCells, kNarrowCellsQ8, kCellBall, kNarrowBall).
+CELL_CHUNK, NARROW_CELLS, NARROW_CELLS_Q8, CELL_BALL, NARROW_BALL = 131072, 16384, 13680, 5, 16
+
+
+def _step_kernels(fp64, Q, nx, ball=None):
+    """Kernels of a step of a solver that launches its stages one by one, and launches per step.  ball: cells that the
+    chi_RET-FM ball reaches on each side (None: chi_SET)."""
+    if fp64 and (nx <= CELL_CHUNK or Q not in (8, 16, 20, 24, 32, 40)):
+        wide = ball is not None and ball > CELL_BALL  # densities and their average before each stage
+        return "fdlb_cell_kernel, fdlb_pair_kernel", 3 * (2 * -(-nx // CELL_CHUNK) + (2 if wide else 0))
+    limit = NARROW_CELLS_Q8 if Q == 8 and ball is None else NARROW_CELLS
+    if not fp64 and nx <= limit and (ball is None or ball <= NARROW_BALL):
+        return "fdlb_narrow_kernel", 3
+    return "fdlb_stage_kernel", 3 if ball is None else 6
+
+
 def _stepping(q, s, steps):
     """The kernel a solver's step calls launch, and how many launches `steps` steps in one call take."""
     per = s.steps_per_launch()
     if per > 0:
         return "fdlb_run_kernel", -(-steps // per)
-    return "fdlb_stage_kernel", 3 * steps
+    kern, launches = _step_kernels(s.precision == q.QL_FP64, s.Q, s.nx)
+    return kern, launches * steps
 
 
 _LAUNCH = {"auto": lambda q: q.QL_LAUNCH_AUTO, "run": lambda q: q.QL_LAUNCH_RUN,
@@ -814,7 +833,8 @@ def run_standing_shock(args):
     steps = sum(r["steps"] for r in rows)
     line = {"metric": "time to steady profile", "value": sum(r["wall_s"] for r in rows if r["precision"] == "fp64"),
             "unit": "s", "n_gpus": 1, "steps": steps, "warmup": 0, "higher_is_better": False, "scaling": "weak",
-            "vs_baseline": None, "dtype": "f64", "data": "synthetic", "gpu_launches": 3 * steps,
+            "vs_baseline": None, "dtype": "f64", "data": "synthetic",
+            "gpu_launches": sum(r["steps"] * _step_kernels(r["precision"] == "fp64", 32, 4096)[1] for r in rows),
             "config": {"workload": "standing_shock_M1.4_nx4096_Q32", "length_l0": 128, "tol_fp64": 1e-9,
                        "tol_fp32": 1e-8, "max_steps": args.shock_steps,
                        "value": "sum of the FP64 runs' times, solver creation to the last residual check"},
@@ -878,7 +898,7 @@ def run_inviscid(args):
                                         np.abs(fields["fp64"][k]).max()) for k in ("rho", "u", "T", "P")}
     line = {"metric": "time to solution", "value": rows[0]["step_loop_s"], "unit": "s", "n_gpus": 1, "steps": steps,
             "warmup": 3, "higher_is_better": False, "scaling": "weak", "vs_baseline": None, "dtype": "f64",
-            "data": "synthetic", "gpu_launches": 3 * steps,
+            "data": "synthetic", "gpu_launches": steps * _step_kernels(True, Q, nx)[1],
             "config": {"workload": "near_inviscid_shock_tube", "length": L, "nx": nx, "Q": Q, "sigma": sigma, "dt": dt,
                        "denseness": El, "chi": "SET", "t_end": t,
                        "value": "FP64 step loop on CUDA events; FP32 in rows"},
@@ -949,9 +969,13 @@ def run_paper_table(args):
             except q.QLError as e:
                 row["fp32"] = {"error": str(e)}
         rows.append(row)
-    # stepping kernels per step (graph nodes): tiled, 3 stages + 3 ball averages; generic path, 4 per stage
-    launches = sum(r["steps"] * (6 if r["path"] == "tiled" else 12) * (2 if "fp32" in r else 1)
-                   for r in rows if "steps" in r)
+    launches = 0
+    for r in rows:
+        if "steps" in r:
+            dx = L / r["nx"]
+            W = max(0, math.ceil(r["sigma"] / dx - 0.5))  # the ball of radius sigma
+            launches += r["steps"] * sum(_step_kernels(fp64, r["Q"], r["nx"], W)[1]
+                                         for fp64 in ((True, False) if "fp32" in r else (True,)))
     line = {"metric": "time to solution", "value": sum(r.get("time_to_solution_s", float("nan")) for r in rows),
             "unit": "s", "gpu_launches": launches,
             "n_gpus": 1, "steps": nsteps, "warmup": 3, "higher_is_better": False, "scaling": "weak",
