@@ -829,7 +829,10 @@ def run_standing_shock(args):
     rows = []
     for El in (0.05, 0.1, 0.2):
         rows.append(_shock_to_steady(q, inputs, 1.4, El, q.QL_FP64, args.shock_steps, 1e-9))
-        rows.append(_shock_to_steady(q, inputs, 1.4, El, q.QL_FP32, args.shock_steps, 1e-8))
+        try:  # the FP32 equilibrium of the densest gas's hot side is too ill-conditioned to run on
+            rows.append(_shock_to_steady(q, inputs, 1.4, El, q.QL_FP32, args.shock_steps, 1e-8))
+        except q.QLError as e:
+            rows.append({"denseness": El, "mach": 1.4, "precision": "fp32", "steps": 0, "error": str(e)})
     steps = sum(r["steps"] for r in rows)
     line = {"metric": "time to steady profile", "value": sum(r["wall_s"] for r in rows if r["precision"] == "fp64"),
             "unit": "s", "n_gpus": 1, "steps": steps, "warmup": 0, "higher_is_better": False, "scaling": "weak",

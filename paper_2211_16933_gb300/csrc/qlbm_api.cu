@@ -608,8 +608,9 @@ static void record_step_graph(ql_ctx *c, int cur)
 // QL_LAUNCH_AUTO for domains of 1 to kRunAutoWaves times as many tiles as the
 // GPU holds CTAs.  Measured on the Sod tube, Q = 32, against per-stage
 // launches: 0.70x the step time at 2^17 cells (1.2 waves of CTAs per stage),
-// 0.92x at 2^19 (4.6 waves), 1.02x at 2^21 (18.5 waves), 1.04x at 2^22; 1.10x
-// at 2^13 and 2^15 (fewer tiles than CTA slots).  Never with fault.
+// 0.92x at 2^19 (4.6 waves), 1.02x at 2^21 (18.5 waves), 1.04x at 2^22; 1.11x
+// at 2^15 (fewer tiles than CTA slots) and 2.3x at 2^13, where the stages are
+// fdlb_narrow_kernel's.  Never with fault.
 constexpr int64_t kRunAutoWaves = 8;
 static bool runs_whole(const ql_ctx *c)
 {
