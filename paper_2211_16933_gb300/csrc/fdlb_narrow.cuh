@@ -77,17 +77,23 @@ __global__ void __launch_bounds__(kThreads, 2) fdlb_narrow_kernel(NarrowArgs s)
         // flight.  The ball's weights (one FP64 conversion each) and densities go through shared memory: with
         // each thread fetching and converting all of its own, balls of 8 and 16 cells were slower than on
         // tiles with the average as a launch of its own (us per step; tiles, each its own, this: Q = 8, 16384 cells, 16 cells:
-        // 24.6, 52.7, 24.5; Q = 20, 5000 cells, 8 cells: 35.0, 30.8, 18.4).
+        // 24.6, 52.7, 23.5; Q = 20, 5000 cells, 8 cells: 34.8, 30.8, 18.5).  A ball within its cell has one
+        // weight and needs no trip through shared memory (balls of one cell are faster with it).
         const int c = t - (kThreads - 64), W = s.f.W;
         const Real *n = static_cast<const Real *>(s.f.n);
-        const double weight = s.f.K[min(c, 2 * W)];  // in flight beside the densities
-        for (int e = c; e < SEG + 2 * W; e += 64) s_bn[e] = fm_density<Real>(s.f, n, i0 - kHalo - W + e);
-        if (c <= 2 * W) s_bk[c] = Real(weight);
-        asm volatile("bar.sync 1, 64;" ::: "memory");
-        if (c < SEG) {
-            Real nbar = 0.f;
+        Real nbar = 0.f;
+        if (W == 0) {
+            if (c < SEG) nbar = fma_(Real(s.f.K[0]), fm_density<Real>(s.f, n, i0 - kHalo + c), nbar);
+        } else {
+            const double weight = s.f.K[min(c, 2 * W)];  // in flight beside the densities
+            for (int e = c; e < SEG + 2 * W; e += 64) s_bn[e] = fm_density<Real>(s.f, n, i0 - kHalo - W + e);
+            if (c <= 2 * W) s_bk[c] = Real(weight);
+            asm volatile("bar.sync 1, 64;" ::: "memory");
+            if (c < SEG)
 #pragma unroll 4
-            for (int d = 0; d <= 2 * W; ++d) nbar = fma_(s_bk[d], s_bn[c + d], nbar);
+                for (int d = 0; d <= 2 * W; ++d) nbar = fma_(s_bk[d], s_bn[c + d], nbar);
+        }
+        if (c < SEG) {
             const Real chi = chi_of_nbar_(a, nbar);
             s_chi[c] = chi;
             s_lnchi[c] = log_(chi);
