@@ -45,15 +45,15 @@ __device__ __forceinline__ int64_t i64_mantissa_(double x, int e)
 // The same as fixed point, bit 59 the leading bit of exponent field E >= e, E >= 1.
 __device__ __forceinline__ int64_t i64_fix_(int64_t m, int e, int E) { return m >> min(E - max(e, 1) + 3, 63); }
 
-// double(Q) rounded to nearest (ties away), |Q| < 2^62; the conversion instruction
+// Q 2^-low rounded to nearest (ties away), |Q| < 2^62, 0 <= low < 900; the conversion instruction
 // occupies the FP64 pipe for about 100 cycles per warp, this about 30 issue slots.
-__device__ __forceinline__ double i64_to_double_(int64_t Q)
+__device__ __forceinline__ double i64_to_double_(int64_t Q, int low)
 {
     uint64_t q = uint64_t(Q < 0 ? -Q : Q);
     const int sh = min(__clzll(int64_t(q)), 64) - 1;
     q = (q << sh) + 0x200;  // leading bit 62, or 63 after a carry (which the addition below puts in the exponent)
     const uint64_t m = q >> 10;
-    const uint32_t hi = uint32_t(m >> 32) + (uint32_t(1084 - sh) << 20);
+    const uint32_t hi = uint32_t(m >> 32) + (uint32_t(1084 - sh - low) << 20);
     return __hiloint2double(Q == 0 ? 0 : int(hi | (uint32_t(Q >> 32) & 0x80000000u)), Q == 0 ? 0 : int(uint32_t(m)));
 }
 
@@ -161,11 +161,12 @@ __device__ __forceinline__ void weno5_faces_i64(const double (&a)[N], const doub
 #pragma unroll
     for (int k = 0; k < N; ++k) {
         const int64_t X = int64_t(x0[k] + uint64_t(__mul64hi(d[k] << 20, int64_t(x0[k] >> 1)) >> 16));
-        // Q = 6 (h - f0) 2^(1079 - T - n): a sixth of the unit, by its exponent
+        // Q = 6 (h - f0) 2^(1079 - T - n): a sixth of the unit, by its exponent, which is kept in the normal
+        // range (T + n is -2 at the least; below 60 only where differences are below 2^-962, or zero)
         const int64_t Q = __mul64hi(Nm[k], X);
-        const int unit = T[k] + n[k] >= 60 ? 0x3FD55555 + ((T[k] + n[k] - 1080) << 20) : 0;
+        const int m = T[k] + n[k], low = max(60 - m, 0), unit = 0x3FD55555 + ((m + low - 1080) << 20);
         const bool nan = max(max(E[0][k], E[1][k]), E[2][k]) == 0x7FF;
-        h[k] = fma(i64_to_double_(Q), __hiloint2double(nan ? 0x7FF80000 : unit, 0x55555555), f0[k]);
+        h[k] = fma(i64_to_double_(Q, low), __hiloint2double(nan ? 0x7FF80000 : unit, 0x55555555), f0[k]);
     }
 }
 __device__ __forceinline__ double weno5_face_i64(double a, double b, double g, double c, double f0)

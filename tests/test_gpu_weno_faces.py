@@ -98,3 +98,11 @@ def _steep_rows():
 @pytest.mark.parametrize("repeat", [1, 250])
 def test_steep_rows_keep_the_relative_precision_of_small_values(gpu, repeat):
     _check_advection(gpu, _steep_rows(), 8, repeat)
+
+
+@pytest.mark.parametrize("repeat", [1, 300])
+def test_differences_near_the_smallest_normal_number(gpu, repeat):
+    """Tails of 1e-300 and 1e-305, alone and beside a value of 1: their differences' unit of 2^-59 is below the normal range."""
+    rng = np.random.default_rng(29)
+    u = lambda n: 1.0 + rng.uniform(0, 1, n)
+    _check_advection(gpu, np.concatenate([1e-300 * u(200), u(20), 1e-305 * u(200), u(20)]), 8, repeat)
