@@ -372,6 +372,8 @@ ql_status ql_closure_create(const ql_closure_desc *desc, const ql_opts *opts, ql
 /* Device arrays: x [B][positions][in_channels] f32, y [B][positions][out_channels]
  * f32 (physical units), periodic [B] int32 (nonzero: periodic padding at the
  * ends, zero: the end values are replicated).  1 <= B <= max_batch.  Asynchronous on the stream.
+ * A kernel that gives up a bounded wait is reported by the next call that reads the error word
+ * (ql_closure_gradients or ql_closure_train_step with a loss, ql_closure_train_steps).
  * y may overlap x and periodic (an overlap other than y in the place of x with as many channels
  * takes the kernels per layer, about half as fast). */
 ql_status ql_closure_forward(ql_closure *c, const float *x, const int32_t *periodic, int64_t B, float *y);
